@@ -80,11 +80,17 @@ typedef struct {
   int max_cycles;   /* cap on cycles (refinement steps for precision 1, 2)    */
   int min_coarse;   /* stop coarsening below this many grid nodes (Sec. 5: 10) */
   int batch;        /* B: right-hand sides solved together                      */
-  int coarse_nodes; /* levels with at most this many grid nodes (and all below
-                       them) run inside one launch per visit; 0 = never       */
-  int coarse_mode;  /* that launch: 0 = one CTA per right-hand side,
-                       1 = a cooperative grid of all co-resident CTAs with
-                       bounded grid-wide barriers (MG_ETIMEOUT if one gives up) */
+  int coarse_nodes; /* the small levels (and all below them) run inside one
+                       launch: with coarse_mode 0 the levels with at most this
+                       many grid nodes per thread block of the launch (up to
+                       16 blocks per right-hand side) that fit in the blocks'
+                       shared memory, with coarse_mode 1 the levels with at
+                       most this many grid nodes; 0 = never                  */
+  int coarse_mode;  /* that launch: 0 = one thread-block cluster per right-hand
+                       side, all of the first level's visits of a cycle in
+                       one launch; 1 = a cooperative grid of all co-resident
+                       CTAs with bounded grid-wide barriers, one launch per
+                       visit (MG_ETIMEOUT if one gives up)                    */
   int fuse;         /* 1 = fused halo-tile kernels: residual + restriction in
                        one pass, fine-level Jacobi sweeps up to 4 per pass;
                        0 = one kernel per step (same results)                  */

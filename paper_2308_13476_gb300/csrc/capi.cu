@@ -14,6 +14,7 @@
 #include "../../include/helmmg.h"
 #include "internal.h"
 #include "ragged_api.h"
+#include "sstep.cuh"
 
 using namespace hmg;
 
@@ -116,11 +117,13 @@ struct mg_ctx {
   cudaGraphExec_t gexec = nullptr;
   cudaGraph_t graph = nullptr;
   std::vector<void*> allocs;
-  int lc = 1 << 30;                  // first level run by the coarse-cycle interpreter
+  int lc = 1 << 30;                  // first level run by the coarse-cycle launch
   int coop_grid = 0;                 // > 0: cooperative interpreter with this many blocks
   CoopCtl coop{};
-  CoarsePlan<double> plan64;
+  CoarsePlan<double> plan64;         // cooperative interpreter (coop_grid > 0)
   CoarsePlan<float> plan32;
+  ClArgs<double> cl64{};             // cluster launch (coop_grid == 0)
+  ClArgs<float> cl32{};
   long long graph_kernels = 0;     // kernel nodes in the cycle graph
   long long last_launches = 0, last_graphs = 0;
   int done = 0;                    // cycles of the current solve
@@ -238,6 +241,9 @@ static OpView<float> op32(const mg_ctx* c, int l) {
 template <class T> static OpView<T> opT(const mg_ctx* c, int l);
 template <> OpView<double> opT<double>(const mg_ctx* c, int l) { return op64(c, l); }
 template <> OpView<float> opT<float>(const mg_ctx* c, int l) { return op32(c, l); }
+template <class T> static ClArgs<T>& clargs(mg_ctx* c);
+template <> ClArgs<double>& clargs<double>(mg_ctx* c) { return c->cl64; }
+template <> ClArgs<float>& clargs<float>(mg_ctx* c) { return c->cl32; }
 template <class T> static std::vector<LevelVec<T>>& vecs(mg_ctx* c);
 template <> std::vector<LevelVec<double>>& vecs<double>(mg_ctx* c) { return c->v64; }
 template <> std::vector<LevelVec<float>>& vecs<float>(mg_ctx* c) { return c->v32; }
@@ -301,8 +307,8 @@ template <class T> struct Emit {
   mg_ctx* c;
   cudaStream_t s;
   std::vector<cx<T>*> cur, oth;
-  int lc;                        // first level run by the coarse-cycle interpreter
-  const CoarsePlan<T>* plan;
+  int lc;                        // first level run by the coarse-cycle launch
+  const CoarsePlan<T>* plan;     // its schedule in the cooperative interpreter
   // complex64 cycle of the FP64 refinement: the FP64 iterate that the
   // level-0 post-smoothing's last GMRES(3) update adds the cycle's result to
   // (the fused refinement update); null: the caller adds it
@@ -341,12 +347,12 @@ template <class T> struct Emit {
 
   void cycle(int l) {
     const int L = c->nlev;
-    if (l >= lc) {   // one visit of the sub-cycle below, in one launch
+    if (l >= lc) {   // the sub-cycle below in one launch (cluster: all of the level's visits)
       if (c->coop_grid > 0)
         launch_cycle_coop<T>(plan->levels, c->nlev, plan->steps, plan->nsteps, c->cinv, c->ncoarse, c->active,
                              c->B, c->coop_grid, c->coop, s);
       else
-        launch_coarse_cycle<T>(plan->levels, plan->steps, plan->nsteps, c->cinv, c->ncoarse, c->B, c->active, s);
+        launch_cluster_cycle<T>(clargs<T>(c), c->B, s);
       return;
     }
     if (l == L - 1) {
@@ -370,6 +376,8 @@ template <class T> struct Emit {
     }
     if (l + 1 == L - 1 && lc > l + 1) {
       coarse_solve(l + 1);
+    } else if (l + 1 >= lc && c->coop_grid == 0) {
+      cycle(l + 1);   // the cluster launch starts from x = 0 and makes all visits
     } else {
       cudaMemsetAsync(cur[l + 1], 0, sizeof(cx<T>) * (size_t)gc.vstride * c->B, s);
       zx[l + 1] = 1;
@@ -475,6 +483,101 @@ template <class T> static cudaError_t build_plan(mg_ctx* c, int lc, CoarsePlan<T
   return cudaMemcpy(P.steps, pl.steps.data(), sizeof(CStep) * P.nsteps, cudaMemcpyHostToDevice);
 }
 
+// The cluster launch's schedule and layout: the recursion of Emit::cycle from
+// level lc on, all of that level's visits (the cycle index times, once on the
+// fine level); false if the levels do not fit on chip.
+template <class T> static bool cluster_plan(mg_ctx* c, int lc, int C, std::vector<ClLev<T>>& lv,
+                                            std::vector<ClStep>& steps, ClArgs<T>& a) {
+  const int L = c->nlev;
+  lv.assign(L - lc, ClLev<T>{});
+  for (int l = lc; l < L; ++l) {
+    ClLev<T>& d = lv[l - lc];
+    const OpView<T> op = opT<T>(c, l);
+    d.nx = c->lev[l].g.nx;
+    d.ny = c->lev[l].g.ny;
+    d.kind = op.kind;
+    d.scale = (T)ss_scale(c->h, l);
+    d.sigma = (T)ss_sigma(op.kind);
+    d.w0 = (T)c->xw.w0;
+    d.w1 = (T)c->xw.w1;
+    d.w2 = (T)c->xw.w2;
+    d.c0 = op.c0;
+    d.kf = op.kf;
+    d.st = op.st;
+    d.dinv = op.dinv;
+    d.plane = op.plane;
+    d.gx = op.gx;
+    d.wx = op.wx;
+    d.hy = op.hy;
+    d.wy = op.wy;
+  }
+  if (!cluster_layout<T>(lv, C, c->opt.smoother == 1, c->ncoarse, a)) return false;
+  std::vector<char> z(L, 0);
+  // x of level lc is zero on entry but for the FP64 path's fine level, where it is the iterate
+  a.x_zero = lc > 0 || c->opt.precision > 0 || c->opt.krylov > 0;
+  z[lc] = a.x_zero != 0;
+  steps.clear();
+  auto smooth = [&](int l, int nu) {
+    if (nu <= 0) return;
+    steps.push_back(ClStep{c->opt.smoother == 0 ? CL_JACOBI : CL_GMRES, l - lc, nu, z[l]});
+    z[l] = 0;
+  };
+  auto cycle = [&](auto&& self, int l) -> void {
+    if (l == L - 1) {
+      steps.push_back(ClStep{CL_COARSE, l - lc, 0, 0});
+      return;
+    }
+    smooth(l, c->opt.nu_pre);
+    steps.push_back(ClStep{CL_RESTRICT, l - lc, 0, 0});
+    z[l + 1] = 1;
+    const int visits = l + 1 == L - 1 ? 1 : c->opt.cycle;
+    for (int q = 0; q < visits; ++q) self(self, l + 1);
+    steps.push_back(ClStep{CL_PROLONG, l - lc, 0, 0});
+    z[l] = 0;
+    smooth(l, c->opt.nu_post);
+  };
+  const int visits = lc == 0 || lc == L - 1 ? 1 : c->opt.cycle;
+  for (int q = 0; q < visits; ++q) cycle(cycle, lc);
+  return true;
+}
+
+template <class T> static cudaError_t build_cluster(mg_ctx* c, int lc, const std::vector<ClLev<T>>& lv,
+                                                    const std::vector<ClStep>& steps, ClArgs<T>& a) {
+  ClLev<T>* dl;
+  ClStep* ds;
+  cudaError_t e;
+  if ((e = dalloc(c, (void**)&dl, sizeof(ClLev<T>) * lv.size()))) return e;
+  if ((e = dalloc(c, (void**)&ds, sizeof(ClStep) * steps.size()))) return e;
+  if ((e = cudaMemcpy(dl, lv.data(), sizeof(ClLev<T>) * lv.size(), cudaMemcpyHostToDevice))) return e;
+  if ((e = cudaMemcpy(ds, steps.data(), sizeof(ClStep) * steps.size(), cudaMemcpyHostToDevice))) return e;
+  a.lev = dl;
+  a.steps = ds;
+  a.nsteps = (int)steps.size();
+  a.inv = c->cinv;
+  a.active = c->active;
+  a.g = c->lev[lc].g;
+  a.b = vecs<T>(c)[lc].b;
+  a.x = vecs<T>(c)[lc].x;
+  return cudaSuccess;
+}
+
+// The first level of the coarse-cycle launch: the cluster takes every level
+// with at most coarse_nodes nodes per block of the cluster that fits on chip.
+template <class T> static cudaError_t choose_cluster(mg_ctx* c) {
+  const int C = cluster_size<T>(c->B);
+  if (C < 1) return cudaSuccess;   // every level as grid-wide kernels
+  std::vector<ClLev<T>> lv;
+  std::vector<ClStep> steps;
+  for (int l = 0; l < c->nlev; ++l) {
+    if (c->lev[l].plane > (long long)c->opt.coarse_nodes * C) continue;
+    ClArgs<T>& a = clargs<T>(c);
+    if (!cluster_plan<T>(c, l, C, lv, steps, a)) continue;
+    c->lc = l;
+    return build_cluster<T>(c, l, lv, steps, a);
+  }
+  return cudaSuccess;
+}
+
 // One FP64 cycle followed by the stopping test (graph body of the FP64 path).
 static void emit_fp64_iteration(mg_ctx* c, cudaStream_t s) {
   Emit<double> e{c, s, {}, {}, c->lc, &c->plan64};
@@ -497,7 +600,8 @@ static void emit_mixed_iteration(mg_ctx* c, cudaStream_t s) {
   const bool fused = c->opt.precision == 1 && c->opt.smoother == 1 && c->opt.nu_post > 0 && c->lc > 0 &&
                      c->nlev > 1;
   if (fused) e.outer0 = c->v64[0].x;
-  cudaMemsetAsync(c->v32[0].x, 0, sizeof(float2) * (size_t)g0.vstride * c->B, s);
+  if (c->lc > 0 || c->coop_grid > 0)   // the cluster launch starts from x = 0
+    cudaMemsetAsync(c->v32[0].x, 0, sizeof(float2) * (size_t)g0.vstride * c->B, s);
   e.zx[0] = 1;
   e.cycle(0);
   if (c->opt.precision == 2) {
@@ -665,22 +769,20 @@ template <class T> struct EmitR {
     else gmres_smooth_kron_rag<T>(v, nu, s);
   }
 
-  void cycle(int l, const std::vector<int>& S) {
+  // visit: the index among the level's visits from the level above
+  void cycle(int l, const std::vector<int>& S, int visit = 0) {
     std::vector<int> G, I;
     for (int p : S) (l >= q(p)->lc ? I : G).push_back(p);
-    if (!I.empty()) {   // one visit of each one's coarse sub-cycle, beside the deeper work of the others
-      std::vector<RagCoarse<T>> v;
-      for (int p : I) {
-        mg_ctx* h = q(p);
-        const CoarsePlan<T>* pl = sizeof(T) == 8 ? (const CoarsePlan<T>*)&h->plan64 : (const CoarsePlan<T>*)&h->plan32;
-        v.push_back(RagCoarse<T>{pl->levels, pl->steps, pl->nsteps, h->cinv, h->ncoarse, h->active});
-      }
+    if (visit > 0) I.clear();   // the cluster launch of the first visit made them all
+    if (!I.empty()) {   // each one's coarse sub-cycle, beside the deeper work of the others
+      std::vector<ClArgs<T>> v;
+      for (int p : I) v.push_back(clargs<T>(q(p)));
       if (G.empty()) {
-        launch_coarse_cycle_rag<T>(v, s);
+        launch_cluster_cycle_rag<T>(v, s);
       } else {
         cudaEventRecord(c->cfork[l], s);
         cudaStreamWaitEvent(c->cstreams[l], c->cfork[l], 0);
-        launch_coarse_cycle_rag<T>(v, c->cstreams[l]);
+        launch_cluster_cycle_rag<T>(v, c->cstreams[l]);
         cudaEventRecord(c->cjoin[l], c->cstreams[l]);
       }
     }
@@ -706,7 +808,7 @@ template <class T> struct EmitR {
     }
     launch_resid_restrict_rag<T>(xf, c->sub[0]->xw, s);
     launch_zero_rag<T>(zv, s);
-    for (int g = 0; g < c->opt.cycle; ++g) cycle(l + 1, G);
+    for (int g = 0; g < c->opt.cycle; ++g) cycle(l + 1, G, g);
     for (size_t k = 0; k < G.size(); ++k) xf[k].rc = cur(G[k], l + 1);   // the coarse correction
     launch_prolong_add_rag<T>(xf, c->sub[0]->xw, s);
     smooth(l, G, c->opt.nu_post);
@@ -1010,29 +1112,30 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
       }
     }
   }
-  // coarse-cycle interpreter: every level from the first one with at most
-  // opt.coarse_nodes nodes down to the coarsest grid
+  // the coarse-cycle launch: the small levels down to the coarsest grid as one
+  // cluster per right-hand side, or (coarse_mode 1) every level from the first
+  // one with at most coarse_nodes nodes on a cooperative grid
   c->lc = 1 << 30;
-  if (o.coarse_nodes > 0)
-    for (int l = 0; l < c->nlev; ++l)
-      if (c->lev[l].plane <= o.coarse_nodes) {
-        c->lc = l;
-        break;
-      }
   CK(cudaStreamSynchronize(s));
-  if (c->lc < c->nlev) {
-    if (!mixed) CK(build_plan<double>(c, c->lc, c->plan64));
-    else CK(build_plan<float>(c, c->lc, c->plan32));
-    if (o.coarse_mode == 1 && c->nlev <= COOP_MAXLEV) {   // cooperative grid: all co-resident blocks, split evenly over the RHS
-      const int gmax = mixed ? coop_max_blocks<float>(c->ncoarse) : coop_max_blocks<double>(c->ncoarse);
-      if (gmax >= c->B) {
-        c->coop_grid = (gmax / c->B) * c->B;
-        CK(dalloc(c, (void**)&c->coop.bar, sizeof(unsigned) * 2));
-        CK(dalloc(c, (void**)&c->coop.partial, sizeof(double) * (size_t)c->coop_grid * NVMAX));
-        c->coop.err = c->n_active + 1;
-        c->coop.spin_limit = 1LL << 22;
-      }
+  if (o.coarse_nodes > 0 && o.coarse_mode == 1 && c->nlev <= COOP_MAXLEV) {   // all co-resident blocks, split evenly over the RHS
+    for (int l = 0; l < c->nlev && c->lc >= c->nlev; ++l)
+      if (c->lev[l].plane <= o.coarse_nodes) c->lc = l;
+    const int gmax = c->lc >= c->nlev ? 0 : mixed ? coop_max_blocks<float>(c->ncoarse) : coop_max_blocks<double>(c->ncoarse);
+    if (gmax >= c->B) {
+      if (!mixed) CK(build_plan<double>(c, c->lc, c->plan64));
+      else CK(build_plan<float>(c, c->lc, c->plan32));
+      c->coop_grid = (gmax / c->B) * c->B;
+      CK(dalloc(c, (void**)&c->coop.bar, sizeof(unsigned) * 2));
+      CK(dalloc(c, (void**)&c->coop.partial, sizeof(double) * (size_t)c->coop_grid * NVMAX));
+      c->coop.err = c->n_active + 1;
+      c->coop.spin_limit = 1LL << 22;
+    } else {
+      c->lc = 1 << 30;
     }
+  }
+  if (o.coarse_nodes > 0 && c->coop_grid == 0) {
+    if (!mixed) CK(choose_cluster<double>(c));
+    else CK(choose_cluster<float>(c));
   }
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(s));

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace hmg {
@@ -204,9 +206,8 @@ template <class T> void gmres_smooth_kron(const Grid& g, const OpView<T>& op, cx
 template <class T> void launch_kron_residual(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                              cx<T>* r, int B, const int* active, int kron_ch, cudaStream_t s);
 
-// Single-CTA coarse-cycle interpreter (coarse.cu).  One CTA per RHS walks a
-// host-recorded list of steps over the levels lc..L-1.
-constexpr int CTA_THREADS = 512;
+// Steps of the small levels' part of a cycle, walked by the cooperative
+// interpreter (coop.cu).
 enum { C_JACOBI = 0, C_GMRES = 1, C_RESTRICT = 2, C_ZERO = 3, C_COARSE = 4, C_PROLONG = 5, C_COPY = 6 };
 template <class T> struct CLevel {
   Grid g;
@@ -231,8 +232,55 @@ struct CStep {
   void* p0;                 // iterate of `level` (in place), or source
   void* p1;                 // destination (Jacobi, copy) or coarse correction (prolong)
 };
-template <class T> void launch_coarse_cycle(const CLevel<T>* levels, const CStep* steps, int nsteps,
-                                            const double2* inv, int N, int B, const int* active, cudaStream_t s);
+
+// Coarse-cycle launch (cluster.cu): the levels lc..L-1 of one right-hand side
+// in the shared memory of a cluster of C blocks, which walks a host-recorded
+// list of steps.
+constexpr int CL_MAXC = 16;      // blocks per cluster
+constexpr int CL_MINROWS = 3;    // rows per block at least (the largest operator radius)
+constexpr int CL_NV = 16;        // values of a cluster-wide sum
+enum { CL_JACOBI = 0, CL_GMRES = 1, CL_RESTRICT = 2, CL_COARSE = 3, CL_PROLONG = 4 };
+struct ClStep {
+  int op, level, arg, zero;   // level: counted from lc; arg: sweeps or steps; zero: x is zero on entry
+};
+template <class T> struct ClLev {
+  int nx, ny, n1, rp;         // intervals, nodes per row, rows per block
+  int kind;                   // as OpView::kind
+  unsigned magic;             // q / n1 = umulhi(q, magic) for the slab's nodes
+  int ox, ob, od;             // shared memory (elements): iterate, right-hand side, inverse diagonal (-1: none)
+  int ogx, owx, ohy, owy;     // Kronecker factors: x rows transposed to [2R+1][n1], the slab's y rows
+  T scale, sigma;             // s-step basis (sstep.cuh)
+  T w0, w1, w2;               // transfers between this level and the next (Xfer)
+  Op0Consts<T> c0;
+  const T* kf;
+  const cx<T>* st;
+  const cx<T>* dinv;
+  long long plane;
+  const cx<T>* gx;
+  const T* wx;
+  const cx<T>* hy;
+  const T* wy;
+};
+template <class T> struct ClArgs {
+  const ClLev<T>* lev;        // nlev levels, device
+  const ClStep* steps;        // device
+  int nlev, nsteps, C;
+  int x_zero;                 // x is zero on entry (not read)
+  int N;                      // coarsest nodes, and the FP64 inverse
+  const double2* inv;
+  const int* active;
+  Grid g;                     // of the first level
+  const cx<T>* b;             // its right-hand side and iterate
+  cx<T>* x;
+  int ou, nu, oX, nX, ored, olev, smem;   // shared memory layout (elements; smem in bytes)
+};
+// Largest cluster (a power of two, at most CL_MAXC) of which B run at once, so
+// that no right-hand side waits for another's visit to end; 0: none.
+template <class T> int cluster_size(int B);
+// Fills the layout of levels (nx, ny, kind set) into lv and a; false if a
+// slab does not fit in a block's shared memory.
+template <class T> bool cluster_layout(std::vector<ClLev<T>>& lv, int C, bool gmres, int N, ClArgs<T>& a);
+template <class T> cudaError_t launch_cluster_cycle(const ClArgs<T>& a, int B, cudaStream_t s);
 
 // Cooperative multi-CTA interpreter (coop.cu): the same steps, all blocks of
 // the GPU, grid-wide barriers between phases.

@@ -65,16 +65,12 @@ void launch_update_mixed_rag(const std::vector<RagOuter>& v, cudaStream_t s);
 void launch_resid_cast_stop_rag(const std::vector<RagOuter>& v, int count, cudaStream_t s);
 void launch_resnorm_stop_rag(const std::vector<RagOuter>& v, int count, cudaStream_t s);
 
-// One visit of each problem's coarse sub-cycle (one CTA per problem).
-template <class T> struct RagCoarse {
-  const CLevel<T>* levels;
-  const CStep* steps;
-  int nsteps;
-  const double2* inv;
-  int N;
-  const int* active;
+// One visit of each problem's coarse sub-cycle (one cluster per problem, all
+// of the same size).
+template <class T> struct ClRag {
+  ClArgs<T> a[32];
 };
-template <class T> void launch_coarse_cycle_rag(const std::vector<RagCoarse<T>>& v, cudaStream_t s);
+template <class T> void launch_cluster_cycle_rag(const std::vector<ClArgs<T>>& v, cudaStream_t s);
 
 // out[p] = the active count of problem p ([0] of its count pair), out[np + p]
 // = its barrier-error flag ([1]).
