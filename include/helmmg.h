@@ -101,11 +101,12 @@ typedef struct {
                        kernels, which then also form the residual before the
                        restriction (needs fuse = 1): 1 = always, 0 = never (the
                        node-parallel kernels; same results to rounding),
-                       -1 = the Kronecker-form levels always, the fine level
-                       when it holds at least 4 M nodes over all right-hand
-                       sides and the other problems of a ragged batch (a row
-                       march keeps each warp on one strip, which needs that
-                       much work to fill the GPU)                           */
+                       -1 = the Kronecker-form levels and the complex64 fine
+                       level always, the complex128 fine level when it holds
+                       at least 4 M nodes over all right-hand sides and the
+                       other problems of a ragged batch (its row march keeps
+                       each warp on one strip, which needs that much work to
+                       fill the GPU)                                         */
   int krylov;       /* 0 = the stand-alone cycle iteration (the paper's method);
                        m in 1..32 = restarted flexible GMRES(m) on the fine
                        operator with one cycle (from zero) as the right

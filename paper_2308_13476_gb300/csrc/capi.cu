@@ -285,9 +285,19 @@ static bool use_march(const mg_ctx* c, int l) {
   return (long long)(g.nx + 1) * (g.ny + 1) * c->B + c->peer_nodes >= (4LL << 20);
 }
 
+// Whether level l's complex64 GMRES(3) steps run as the s-step row marches:
+// the fine level whenever marches are allowed.  They need no size threshold:
+// on one 1025^2 right-hand side a step takes 31 us against the node-parallel
+// kernels' 85 us, at 64 right-hand sides 587 against the Arnoldi marches'
+// 1210 us.
+static bool use_ss_march(const mg_ctx* c, int l) {
+  return c->opt.precision > 0 && c->opt.fuse && c->opt.march != 0 && c->lev[l].kind == 1;
+}
+
+// Returns the vector that holds the smoothed iterate: x, or xt.
 template <class T>
-static void gmres_level(mg_ctx* c, int l, cx<T>* x, const cx<T>* b, int nu, const int* active, cudaStream_t s,
-                        double2* outer = nullptr, bool x_zero = false) {
+static cx<T>* gmres_level(mg_ctx* c, int l, cx<T>* x, cx<T>* xt, const cx<T>* b, int nu, const int* active,
+                          cudaStream_t s, double2* outer = nullptr, bool x_zero = false) {
   const Grid& g = c->lev[l].g;
   const OpView<T> op = opT<T>(c, l);
   GmresBufs gb = vecs<T>(c)[l].gb;
@@ -297,10 +307,20 @@ static void gmres_level(mg_ctx* c, int l, cx<T>* x, const cx<T>* b, int nu, cons
   gb.ev_join = c->ev_join;
   gb.outer = outer;
   gb.x_zero = x_zero;
+  gb.scale = (float)ss_scale(c->h, l);
+  gb.sigma = (float)ss_sigma(op.kind);
+  if constexpr (sizeof(T) == 4) {
+    if (use_ss_march(c, l)) return gmres_smooth_ss_march(g, op, x, xt, b, nu, c->B, active, gb, s);
+  }
   const bool m = use_march(c, l);
-  if (m && op.kind == 1) gmres_smooth_march<T>(g, op, x, b, nu, c->B, active, gb, s);
-  else if (m && op.kind >= 4) gmres_smooth_kron<T>(g, op, x, b, nu, c->B, active, gb, s);
-  else gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
+  if (m && op.kind >= 4) gmres_smooth_kron<T>(g, op, x, b, nu, c->B, active, gb, s);
+  else if constexpr (sizeof(T) == 8) {
+    if (m && op.kind == 1) gmres_smooth_march<T>(g, op, x, b, nu, c->B, active, gb, s);
+    else gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
+  } else {
+    gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
+  }
+  return x;
 }
 
 template <class T> struct Emit {
@@ -336,7 +356,7 @@ template <class T> struct Emit {
         std::swap(cur[l], oth[l]);
       }
     } else {
-      gmres_level<T>(c, l, cur[l], V.b, nu, c->active, s, outer, z);
+      if (gmres_level<T>(c, l, cur[l], oth[l], V.b, nu, c->active, s, outer, z) != cur[l]) std::swap(cur[l], oth[l]);
     }
   }
 
@@ -600,7 +620,9 @@ static void emit_mixed_iteration(mg_ctx* c, cudaStream_t s) {
   const bool fused = c->opt.precision == 1 && c->opt.smoother == 1 && c->opt.nu_post > 0 && c->lc > 0 &&
                      c->nlev > 1;
   if (fused) e.outer0 = c->v64[0].x;
-  if (c->lc > 0 || c->coop_grid > 0)   // the cluster launch starts from x = 0
+  // the cluster launch and the s-step march's first step start from x = 0 without reading it
+  const bool whole = c->lc == 0 && c->coop_grid == 0;
+  if (!whole && !(c->lc > 0 && c->nlev > 1 && c->opt.smoother == 1 && c->opt.nu_pre > 0 && use_ss_march(c, 0)))
     cudaMemsetAsync(c->v32[0].x, 0, sizeof(float2) * (size_t)g0.vstride * c->B, s);
   e.zx[0] = 1;
   e.cycle(0);
@@ -692,7 +714,7 @@ template <class T> static mg_status profile_t(mg_ctx* h, int what, int level, in
       case 1: launch_residual<T>(g, op, V[level].x, V[level].b, V[level].r, h->B, nullptr, s); break;
       case 2: launch_restrict<T>(g, h->lev[level + 1].g, V[level].r, V[level + 1].b, h->B, nullptr, h->xw, s); break;
       case 3: launch_prolong_add<T>(g, h->lev[level + 1].g, V[level + 1].x, V[level].x, h->B, nullptr, h->xw, s); break;
-      case 4: gmres_level<T>(h, level, V[level].x, V[level].b, 1, nullptr, s); break;
+      case 4: gmres_level<T>(h, level, V[level].x, V[level].t, V[level].b, 1, nullptr, s); break;
       default: {   // the last Arnoldi step of a restart cycle (j = m - 1): both passes, every RHS active
         const int j = h->opt.krylov - 1;
         cudaMemcpyAsync(h->active, ones.data(), sizeof(int) * h->B, cudaMemcpyHostToDevice, s);
@@ -754,7 +776,11 @@ template <class T> struct EmitR {
   cudaStream_t s;
   int P() const { return (int)c->sub.size(); }
   mg_ctx* q(int p) const { return c->sub[p]; }
-  cx<T>* cur(int p, int l) const { return vecs<T>(c->sub[p])[l].x; }   // GMRES(3) smoothing keeps x in place
+  bool swapped = false;   // complex64: the fine level's iterate sits in t (an odd number of s-step marches)
+  cx<T>* cur(int p, int l, bool other = false) const {   // other levels' smoothing keeps x in place
+    auto& V = vecs<T>(c->sub[p])[l];
+    return (l == 0 && swapped && q(p)->lc > 0) != other ? V.t : V.x;
+  }
 
   void smooth(int l, const std::vector<int>& G, int nu) {
     if (nu <= 0 || G.empty()) return;
@@ -763,10 +789,24 @@ template <class T> struct EmitR {
       mg_ctx* h = q(p);
       GmresBufs gb = vecs<T>(h)[l].gb;
       gb.kron_ch = h->opt.kron_chunk;
-      v.push_back(RagLevel<T>{h->lev[l].g, opT<T>(h, l), cur(p, l), vecs<T>(h)[l].b, gb, h->active});
+      gb.scale = (float)ss_scale(h->h, l);
+      gb.sigma = (float)ss_sigma(h->lev[l].kind);
+      v.push_back(RagLevel<T>{h->lev[l].g, opT<T>(h, l), cur(p, l), cur(p, l, true), vecs<T>(h)[l].b, gb, h->active});
     }
-    if (l == 0) gmres_smooth_march_rag<T>(v, nu, s, c->side, c->ev_fork, c->ev_join);
-    else gmres_smooth_kron_rag<T>(v, nu, s);
+    if constexpr (sizeof(T) == 4) {
+      if (l == 0) {
+        gmres_smooth_ss_march_rag(v, nu, s);
+        swapped ^= (nu & 1) != 0;
+        return;
+      }
+    }
+    if constexpr (sizeof(T) == 8) {
+      if (l == 0) {
+        gmres_smooth_march_rag<T>(v, nu, s, c->side, c->ev_fork, c->ev_join);
+        return;
+      }
+    }
+ gmres_smooth_kron_rag<T>(v, nu, s);
   }
 
   // visit: the index among the level's visits from the level above
@@ -841,6 +881,7 @@ static void emit_ragged_iteration(mg_ctx* c, cudaStream_t s) {
     launch_zero_rag<float>(zv, s);
     EmitR<float> e{c, s};
     e.cycle(0, e.all());
+    for (int p = 0; p < P; ++p) outer[p].e = e.cur(p, 0);
     launch_update_mixed_rag(outer, s);
     launch_resid_cast_stop_rag(outer, 1, s);
   } else {
@@ -1073,8 +1114,8 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
   for (int l = 0; l < c->nlev; ++l) {
     nblk_max = std::max(nblk_max, node_blocks(c->lev[l].g));
     if (c->lev[l].kind == 1)
-      nblk_max = std::max({nblk_max, gmres_march_blocks(c->lev[l].g, true, c->B),
-                           gmres_march_blocks(c->lev[l].g, false, c->B)});
+      nblk_max = std::max({nblk_max, gmres_march_blocks(c->lev[l].g, c->B),
+                           mixed && gm ? ss_march_blocks(c->lev[l].g, c->B) : 0LL});
     if (c->lev[l].kind >= 4) nblk_max = std::max(nblk_max, kron_march_blocks(c->lev[l].g, c->B));
   }
   CK(dalloc(c, (void**)&c->partial, sizeof(double) * (size_t)nblk_max * c->B * NVMAX));

@@ -126,30 +126,9 @@ template <class T> struct Slab {
   for (int q = B.tid, jl = __umulhi(B.tid, (s).L->magic), i = q - jl * (s).n1; q < (s).nodes; \
        q += NT, jl = __umulhi(q, (s).L->magic), i = q - jl * (s).n1)
 
-// Sums the NV per-thread values over the cluster: a butterfly that halves the
-// number of values each lane carries at every exchange (NV - 1 + (5 - log2
-// NV) adds instead of 5 NV: the FP64 pipe is narrow), the warps' sums in warp
-// order, and the blocks' sums pushed to every block.  After the caller's next
-// cl_sync(), cl_totals() gives the totals.
-template <int NV, class T> __device__ __forceinline__ T lane_sum(T (&v)[NV], int lane) {
-  // NV a power of two <= 32: lane holds value (lane's top log2(NV) bits, reversed by halving) at the end
-  int o = 16;
-#pragma unroll
-  for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const T keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  T t = v[0];
-  for (; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
-// the value index that lane_sum leaves in a lane: the leading log2(NV) lane bits
-template <int NV> __device__ __forceinline__ int lane_value(int lane) { return lane / (32 / NV); }
-
+// Sums the NV per-thread values over the cluster: lane_sum within the warps,
+// the warps' sums in warp order, and the blocks' sums pushed to every block.
+// After the caller's next cl_sync(), cl_totals() gives the totals.
 template <int NV, int NT, class T>
 __device__ __forceinline__ void cl_push_sum(Blk<T>& B, T (&v)[NV]) {
   static_assert(NV <= CL_NV, "record");

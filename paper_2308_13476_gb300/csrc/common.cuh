@@ -18,7 +18,7 @@ constexpr int BX = 32;   // block shape of the node-parallel kernels
 constexpr int BY = 8;
 constexpr int RYMAX = 4; // largest number of grid rows per thread (Grid::ry)
 constexpr int MAXR = 3;  // largest Galerkin stencil radius (7 x 7)
-constexpr int NVMAX = 12; // values per block partial record
+constexpr int NVMAX = 16; // values per block partial record
 
 template <class T> struct cvec;
 template <> struct cvec<double> { using type = double2; };
@@ -368,6 +368,29 @@ template <class T, int R> struct OpK {
     return dinvp[(long long)j * (nx + 1) + i];
   }
 };
+
+// Warp sums of NV values per lane (NV a power of two <= 32): a butterfly that
+// halves the number of values each lane carries at every exchange (NV - 1 +
+// 5 - log2 NV adds and as many shuffles instead of 5 NV).  The sum of value
+// lane_value<NV>(lane) is returned, in every lane of the value's group of 32 /
+// NV lanes.
+template <int NV, class T> __device__ __forceinline__ T lane_sum(T (&v)[NV], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int h = NV / 2; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const T keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  T t = v[0];
+#pragma unroll
+  for (; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+template <int NV> __device__ __forceinline__ int lane_value(int lane) { return lane / (32 / NV); }
 
 // Final stage of the block sums below: value k of the block is the sum of
 // the warps' partial sums sh[k][0..nwarps) added in warp order.  Lane k of

@@ -15,9 +15,9 @@
 //   M2: u2 = s1 A u1 - sum c_l1 u_l       |u2|^2, <u2, u_l>, <u_l, A u2>
 //   M3: u3 = s2 A u2 - sum c_l2 u_l       |u3|^2 (not stored)
 //   then x += sum y_l s_l u_l (g_update).
-// That is 16 vector passes per step.  complex64 steps skip M3: M2 also sums
-// |A u2|^2, and |u3|^2 follows from the Gram form (13 vector passes).  The scalar steps between passes are the
-// same FP64 Gram-matrix updates and Givens solve (gmres.cuh) in the same order
+// That is 16 vector passes per step (complex128; the complex64 cycles take
+// the s-step marches of sstep_march.cu).  The scalar steps between passes are
+// the same FP64 Gram-matrix updates and Givens solve (gmres.cuh) in the same order
 // as the node-parallel version; only the dots of A u_{j+1} are taken before
 // the scale s_{j+1} is known, and scaled afterwards.
 //
@@ -47,207 +47,13 @@
 
 #include "gmres.cuh"
 #include "internal.h"
+#include "march.cuh"
 #include "ragged.cuh"
 #include "ragged_api.h"
 
 namespace hmg {
 
 namespace {
-
-// staging slots per field of a pass with NF input fields
-template <int NF> struct Ring { static constexpr int NS = NF == 1 ? 8 : NF == 2 ? 6 : 4; };
-// shared memory of a pass: the staging ring, and afterwards the [NVMAX][32]
-// doubles of the block reduction
-template <int NF> constexpr int ring_bytes() {
-  return NF * Ring<NF>::NS * 32 * 16 > NVMAX * 32 * 8 ? NF * Ring<NF>::NS * 32 * 16 : NVMAX * 32 * 8;
-}
-
-template <class T> struct MNP { static constexpr int NP = 1; };
-template <> struct MNP<float> { static constexpr int NP = 2; };
-
-template <class T> struct Row { cx<T> v[MNP<T>::NP]; };
-
-template <class T> __device__ __forceinline__ cx<T> zc() { return mk<T>(T(0), T(0)); }
-template <class T> __device__ __forceinline__ Row<T> zrow() {
-  Row<T> r;
-#pragma unroll
-  for (int n = 0; n < MNP<T>::NP; ++n) r.v[n] = zc<T>();
-  return r;
-}
-
-// Asynchronous copy of this lane's 16 bytes of row j (nodes i..) into a
-// shared-memory slot; columns right of the grid are zero-filled (the padded
-// layout makes the two columns left of the grid and the rows -2..ny+2
-// readable zeros).
-template <class T>
-__device__ __forceinline__ void stage_row(uint32_t dst, const cx<T>* __restrict__ s, const Grid& g, int i, int j) {
-  const bool ok = i <= g.nx;
-  const cx<T>* src = s + g.at(ok ? i : 0, j);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void stage_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ Row<float> stage_read(const float4* p) {
-  const float4 q = *p;
-  Row<float> r;
-  r.v[0] = make_float2(q.x, q.y);
-  r.v[1] = make_float2(q.z, q.w);
-  return r;
-}
-__device__ __forceinline__ Row<double> stage_read(const double2* p) {
-  Row<double> r;
-  r.v[0] = *p;
-  return r;
-}
-template <class T> struct SlotT { using type = double2; };
-template <> struct SlotT<float> { using type = float4; };
-
-__device__ __forceinline__ void mstore(float2* __restrict__ d, const Grid& g, int i, int j, const Row<float>& r) {
-  if (i + 1 <= g.nx)
-    *reinterpret_cast<float4*>(d + g.at(i, j)) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
-  else if (i <= g.nx)
-    d[g.at(i, j)] = r.v[0];
-}
-__device__ __forceinline__ void mstore(double2* __restrict__ d, const Grid& g, int i, int j, const Row<double>& r) {
-  if (i <= g.nx) d[g.at(i, j)] = r.v[0];
-}
-
-template <class T> __device__ __forceinline__ cx<T> shfl_up1(cx<T> a) {
-  return mk<T>(__shfl_up_sync(0xffffffffu, a.x, 1), __shfl_up_sync(0xffffffffu, a.y, 1));
-}
-template <class T> __device__ __forceinline__ cx<T> shfl_dn1(cx<T> a) {
-  return mk<T>(__shfl_down_sync(0xffffffffu, a.x, 1), __shfl_down_sync(0xffffffffu, a.y, 1));
-}
-
-// March modes: MD = 1 interior strips (branch-free stencil), MD = 2 edge
-// strips over interior rows (the same stencil, with the boundary row of
-// Op0::apply5 on columns 0 and nx and zero off the grid), MD = 0 everything
-// else (the 3-row bands; every warp on grids of fewer than 7 rows).  MD + 4
-// (modes 0 and 2 only): the same with the second-order absorbing rows of
-// Op0<T, true> on the boundary nodes (interior strips touch none).
-template <int MD> constexpr int MM = MD & 3;
-template <int MD> constexpr bool MA2 = (MD & 4) != 0;
-// Per-warp march context.
-template <class T, int MD> struct MCtx {
-  static constexpr int NP = MNP<T>::NP;
-  Op0<T, MA2<MD>> op;
-  Grid g;
-  int i;       // first node of this lane
-  int j0, j1;  // chunk rows [j0, j1)
-  bool outl;   // the lane's nodes are in the strip's output columns
-
-  // (A v) on row m from rows m-1, m, m+1 of v; zero for nodes outside the
-  // grid.  All lanes must call it (shuffles).
-  __device__ __forceinline__ Row<T> apply(const Row<T>& dn, const Row<T>& c, const Row<T>& up, int m) const {
-    const cx<T> west = shfl_up1<T>(c.v[NP - 1]);
-    const cx<T> east = shfl_dn1<T>(c.v[0]);
-    Row<T> r;
-#pragma unroll
-    for (int n = 0; n < NP; ++n) {
-      const cx<T> xe = n + 1 < NP ? c.v[n + 1 < NP ? n + 1 : 0] : east;
-      const cx<T> xw = n > 0 ? c.v[n > 0 ? n - 1 : 0] : west;
-      const int in = i + n;
-      if (MM<MD> != 0) {   // Op0::apply5, interior case
-        const cx<T> xn = up.v[n], xs = dn.v[n], xp = c.v[n];
-        const int ik = MM<MD> == 2 ? min(max(in, 0), op.nx) : in;   // edge strips: k of an in-grid node
-        const T k = op.kf ? op.kf[m * (op.nx + 1) + ik] : op.c.k;
-        const T d = fma(-k, k, T(4) * op.c.inv_h2);
-        if constexpr (sizeof(T) == 4) {   // the same operations, both components per instruction
-          const float2 sn = add2(add2(xe, xw), add2(xn, xs));
-          r.v[n] = fma2(bc2(d), xp, mul2(bc2(-op.c.inv_h2), sn));
-        } else {
-          const T sr = (xe.x + xw.x) + (xn.x + xs.x), si = (xe.y + xw.y) + (xn.y + xs.y);
-          r.v[n] = mk<T>(fma(d, xp.x, -op.c.inv_h2 * sr), fma(d, xp.y, -op.c.inv_h2 * si));
-        }
-        if (MM<MD> == 2) {   // rows are interior here; columns 0 and nx take the
-                         // boundary row of Op0::apply5, columns off the grid zero
-          const bool bcol = in == 0 || in == op.nx, inside = in >= 0 && in <= op.nx;
-          if (bcol) r.v[n] = op.apply5(xp, xe, xw, xn, xs, in, m);
-          if (!inside) r.v[n] = zc<T>();
-        }
-      } else {
-        r.v[n] = (m >= 0 && m <= op.ny && in >= 0 && in <= op.nx)
-                     ? op.apply5(c.v[n], xe, xw, up.v[n], dn.v[n], in, m)
-                     : zc<T>();
-      }
-    }
-    return r;
-  }
-  // node n of the lane counts in the dots of row m
-  __device__ __forceinline__ bool cnt(int n, int m) const {
-    return outl && (MM<MD> == 1 || i + n <= g.nx) && m >= j0 && m < j1;
-  }
-  __device__ __forceinline__ bool own_row(int m) const { return outl && m >= j0 && m < j1; }
-};
-
-// Register slot of row t + d at unroll phase S (the march starts at t0 = j0 -
-// 2 with phase 0, so row r sits in slot (r - j0 + 2) mod 4).
-template <int S, int D> struct Sl { static constexpr int v = (S + D + 8) & 3; };
-
-// The NF input fields of a pass: shared-memory staging and register rings.
-// Staging slot (f, k) of a lane is at sbase + (f NS + k) 512 bytes.
-template <class T, int MD, int NF> struct MIn {
-  static constexpr int NS = Ring<NF>::NS, AH = NS - 1;   // AH: rows in flight ahead of use
-  MCtx<T, MD> c;
-  const cx<T>* src[NF];
-  uint32_t sbase;   // shared address of this lane's slot 0 of field 0
-  Row<T> F[NF][4];  // register ring: row r in slot (r - j0 + 2) mod 4
-  int t1;           // last row the march reads
-  int sw, sr;       // staging slots of the next row to issue and to read
-
-  __device__ __forceinline__ void issue(int r, int slot) {
-#pragma unroll
-    for (int f = 0; f < NF; ++f) stage_row<T>(sbase + (f * NS + slot) * 32 * 16, src[f], c.g, c.i, r);
-  }
-  // rows t0 .. t0 + AH - 1 in flight, in slots 0 .. AH - 1
-  __device__ __forceinline__ void prime(int t0) {
-#pragma unroll
-    for (int d = 0; d < AH; ++d) {
-      if (t0 + d <= t1) issue(t0 + d, d);
-      stage_commit();
-    }
-    sw = AH;
-    sr = 0;
-  }
-  // row t + AH in flight (into the slot row t - 1 left), row t into the
-  // register ring
-  template <int S> __device__ __forceinline__ void fetch(int t) {
-    if (t + AH <= t1) issue(t + AH, sw);
-    sw = sw + 1 == NS ? 0 : sw + 1;
-    stage_commit();
-    stage_wait<AH>();
-#pragma unroll
-    for (int f = 0; f < NF; ++f)
-      F[f][Sl<S, 0>::v] = stage_read(reinterpret_cast<const typename SlotT<T>::type*>(
-          __cvta_shared_to_generic(sbase + (f * NS + sr) * 32 * 16)));
-    sr = sr + 1 == NS ? 0 : sr + 1;
-  }
-};
-
-// Runs p.step<S>(t) for t = t0..t1, S = (t - t0) mod 4.
-template <class P> __device__ __forceinline__ void march(P& p, int t0, int t1) {
-#pragma unroll 1
-  for (int t = t0; t <= t1; t += 4) {
-    p.template step<0>(t);
-    if (t + 1 > t1) break;
-    p.template step<1>(t + 1);
-    if (t + 2 > t1) break;
-    p.template step<2>(t + 2);
-    if (t + 3 > t1) break;
-    p.template step<3>(t + 3);
-  }
-}
-
-// complex64 steps take the norm of the last Arnoldi vector u3 = A v2 -
-// sum_l h_l2 v_l from the Gram form instead of a fourth pass: with unit
-// v_l the modified Gram-Schmidt steps give |u3|^2 = |A v2|^2 - sum_l
-// |h_l2|^2 exactly, so M2 also sums |A u2|^2 (s_2 A u2 = A v2) and M3 is
-// not run.  complex128 steps keep M3 (their iterates follow the oracle's
-// explicit norm to rounding).
-template <class T> constexpr bool G3 = sizeof(T) == 4;
-template <class T> constexpr int NV2 = G3<T> ? 12 : 11;
 
 // M0 at iteration t: x and b rows t arrive; u0 row t-1 = b - A x formed from
 // x rows t-2..t; A u0 on row t-2.
@@ -366,7 +172,7 @@ template <class T, int MD> struct P2 {
   T s1;
   cx<T> c0, c1;
   Row<T> U[4];
-  T acc[NV2<T>];
+  T acc[11];
   template <int S> __device__ __forceinline__ void step(int t) {
     m.template fetch<S>(t);
     const MCtx<T, MD>& c = m.c;
@@ -406,7 +212,6 @@ template <class T, int MD> struct P2 {
           acc[8] += d1.y;
           acc[9] += d2.x;
           acc[10] += d2.y;
-          if constexpr (G3<T>) acc[11] += abs2<T>(au.v[n]);   // |A u2|^2: u3's norm without M3
         }
     }
   }
@@ -433,50 +238,6 @@ template <class T, int MD> struct P3 {
         acc[0] += abs2<T>(u);
       }
   }
-};
-
-// Per-warp geometry inside one right-hand side.  With band = 1 (grids of at
-// least 7 rows) the interior set is every strip over rows [3, ny-2) in chunks
-// of ch rows: strips [e_lo, e_hi), whose loaded columns hold no boundary
-// column, take the branch-free stencil; the others (the edge strips) take it
-// too and replace it by the boundary row of Op0::apply5 on columns 0 and nx
-// and by zero off the grid (lane-constant choices: their rows are interior).
-// The boundary set is the 3-row bands at the top (rows 0..2) and bottom (rows
-// ny-2..ny) of every strip.  With band = 0 every warp is a boundary warp, in
-// chunks of chb rows from row 0.
-struct MGeo {
-  int nstrips, ny, band, ch, chb;
-  int e_lo, e_hi;   // strips of the interior set without a boundary column
-  int nci;          // chunks per strip over rows [3, ny-2)
-  int ni, nb;       // warps of the interior strips and of the 3-row bands (or of the whole grid)
-  // strip and rows [j0, j1) of warp w of the set
-  // interior strips [e_lo, e_hi), the edge strips outside that range, each
-  // over rows [3, ny-2) in chunks of ch rows
-  __host__ __device__ __forceinline__ int ne() const { return (nstrips - (e_hi - e_lo)) * nci; }
-  template <int MD> __host__ __device__ __forceinline__ void map(int w, int& strip, int& j0, int& j1) const {
-    if (MD != 0) {
-      const int nse = nstrips - (e_hi - e_lo), nsm = MD == 1 ? e_hi - e_lo : nse;
-      const int sidx = w % nsm;
-      strip = MD == 1 ? e_lo + sidx : (sidx < e_lo ? sidx : e_hi + (sidx - e_lo));
-      j0 = 3 + (w / nsm) * ch;
-      j1 = j0 + ch < ny - 2 ? j0 + ch : ny - 2;
-      return;
-    }
-    if (!band) {
-      strip = w % nstrips;
-      j0 = (w / nstrips) * chb;
-      j1 = j0 + chb < ny + 1 ? j0 + chb : ny + 1;
-      return;
-    }
-    strip = w % nstrips;
-    j0 = w < nstrips ? 0 : ny - 2;
-    j1 = j0 + 3;
-  }
-  // first reduction record of a mode's warps: interior, then edge, then the rest
-  template <int MD> __host__ __device__ __forceinline__ int rec0() const {
-    return MD == 1 ? 0 : (MD == 2 ? ni : ni + ne());
-  }
-  __host__ __device__ __forceinline__ int nrec() const { return ni + ne() + nb; }
 };
 
 template <class T> __host__ __device__ constexpr int strip_w() { return 32 * MNP<T>::NP - 4; }
@@ -664,7 +425,7 @@ __device__ __forceinline__ void gm_step2_body(uint3 vblk, Grid g, MGeo mg, Op0<T
   const T s1 = (T)S[G_S + 1];
   const cx<T> c0 = mk<T>((T)(S[G_H + 2 * 1] * S[G_S]), (T)(S[G_H + 2 * 1 + 1] * S[G_S]));
   const cx<T> c1 = mk<T>((T)(S[G_H + 2 * 4] * S[G_S + 1]), (T)(S[G_H + 2 * 4 + 1] * S[G_S + 1]));
-  T acc[NV2<T>];
+  T acc[11];
   __shared__ __align__(16) unsigned char stg[ring_bytes<2>()];
   double* sh = reinterpret_cast<double*>(stg);
   run_pass<P2>(ctx, j1 + 1, stg, acc, [&](auto& p) {
@@ -681,7 +442,6 @@ __device__ __forceinline__ void gm_step2_body(uint3 vblk, Grid g, MGeo mg, Op0<T
       const double s2 = s[G_S + 2];
       const double d[6] = {q[5] * s2, q[6] * s2, q[7] * s2, q[8] * s2, q[9] * s2, q[10] * s2};
       fin_a<2, T>(s, d);
-      if constexpr (G3<T>) fin_b2_gram<T>(s, q[11] * s2 * s2);
     }
   });
 }
@@ -753,32 +513,12 @@ __global__ void __launch_bounds__(32) gm_step3_rag(const __grid_constant__ RagLa
 template <class T> MGeo march_geo(const Grid& g, int B) {
   constexpr int NP = MNP<T>::NP, SW = strip_w<T>();
   MGeo m;
-  m.nstrips = cdiv(g.nx + 1, SW);
-  m.ny = g.ny;
-  m.band = g.ny >= 6;
-  m.chb = 16;
-  m.e_lo = m.e_hi = 0;
-  for (int s = 0; s < m.nstrips; ++s) {
-    const int cs = s * SW - 2;
-    if (cs >= 1 && cs + 32 * NP - 1 <= g.nx - 1) {
-      if (m.e_hi == 0) m.e_lo = s;
-      m.e_hi = s + 1;
-    }
-  }
+  m.fill(g.nx, g.ny, SW, 32 * NP, 2, 3);
   const int inner_rows = g.ny - 5;
   const long long want = 152LL * 48;   // warps to fill the GPU a few times over
   int ch = 64;
   while (ch > 8 && (long long)m.nstrips * cdiv(inner_rows, ch) * B < want) ch /= 2;
-  m.ch = ch;
-  if (m.band) {
-    m.nci = cdiv(inner_rows, ch);
-    m.ni = (m.e_hi - m.e_lo) * m.nci;
-    m.nb = 2 * m.nstrips;
-  } else {
-    m.e_lo = m.e_hi = 0;
-    m.nci = m.ni = 0;
-    m.nb = m.nstrips * cdiv(g.ny + 1, m.chb);
-  }
+  m.chunks(ch);
   return m;
 }
 
@@ -788,9 +528,8 @@ template <class T> MGeo march_geo(const Grid& g, int B) {
 template <class T> void launch_gmres_update(const Grid& g, cx<T>* x, const GmresBufs& gb, int B, const int* active,
                                             cudaStream_t s);
 
-long long gmres_march_blocks(const Grid& g, bool fp64, int B) {
-  const MGeo m = fp64 ? march_geo<double>(g, B) : march_geo<float>(g, B);
-  return (long long)m.nrec();
+long long gmres_march_blocks(const Grid& g, int B) {
+  return march_geo<double>(g, B).nrec();
 }
 
 template <class T>
@@ -847,17 +586,9 @@ void gmres_smooth_march(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<
       pass([&] { gm_step2<T, 1><<<gi, 32, 0, s>>>(g, mg, op, v0, u1, u2, st, P, tk, active); },
            [&] { gm_step2<T, ME><<<ge, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); },
            [&] { gm_step2<T, MB><<<gbd, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); });
-      if constexpr (!G3<T>) {   // complex64: u3's norm came from the Gram form in M2
-        pass([&] { gm_step3<T, 1><<<gi, 32, 0, s>>>(g, mg, op, v0, u1, u2, st, P, tk, active); },
-             [&] { gm_step3<T, ME><<<ge, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); },
-             [&] { gm_step3<T, MB><<<gbd, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); });
-      }
-      if constexpr (sizeof(T) == 4) {
-        if (step == nu - 1 && gb.outer) {
-          launch_gmres_update_outer(g, x, gs, B, active, s);
-          continue;
-        }
-      }
+      pass([&] { gm_step3<T, 1><<<gi, 32, 0, s>>>(g, mg, op, v0, u1, u2, st, P, tk, active); },
+           [&] { gm_step3<T, ME><<<ge, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); },
+           [&] { gm_step3<T, MB><<<gbd, 32, 0, sb>>>(g, mg, opb, v0, u1, u2, st, P, tk, active); });
       launch_gmres_update<T>(g, x, gs, B, active, s);
     }
   };
@@ -907,18 +638,14 @@ void gmres_smooth_march_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStrea
     pass(gm_init_rag<T, 1>, gm_init_rag<T, 2>, gm_init_rag<T, 0>);
     pass(gm_step1_rag<T, 1>, gm_step1_rag<T, 2>, gm_step1_rag<T, 0>);
     pass(gm_step2_rag<T, 1>, gm_step2_rag<T, 2>, gm_step2_rag<T, 0>);
-    if constexpr (!G3<T>) pass(gm_step3_rag<T, 1>, gm_step3_rag<T, 2>, gm_step3_rag<T, 0>);
+    pass(gm_step3_rag<T, 1>, gm_step3_rag<T, 2>, gm_step3_rag<T, 0>);
     launch_gmres_update_rag<T>(v, s);
   }
 }
 
 template void gmres_smooth_march_rag<double>(const std::vector<RagLevel<double>>&, int, cudaStream_t, cudaStream_t,
                                              cudaEvent_t, cudaEvent_t);
-template void gmres_smooth_march_rag<float>(const std::vector<RagLevel<float>>&, int, cudaStream_t, cudaStream_t,
-                                            cudaEvent_t, cudaEvent_t);
 template void gmres_smooth_march<double>(const Grid&, const OpView<double>&, double2*, const double2*, int, int,
                                          const int*, const GmresBufs&, cudaStream_t);
-template void gmres_smooth_march<float>(const Grid&, const OpView<float>&, float2*, const float2*, int, int,
-                                        const int*, const GmresBufs&, cudaStream_t);
 
 }  // namespace hmg

@@ -180,6 +180,7 @@ struct GmresBufs {
   int x_zero;          // x is zero on entry: the first step takes b itself as
                        // u0 = b - A x (no apply, no u0 write; b is read-only
                        // in every pass) and only sums |b|^2 for its norm
+  float scale, sigma;  // complex64 s-step basis of the level (sstep.cuh)
 };
 // The last GMRES(3) update of a complex64 level-0 smoothing fused with the
 // FP64 refinement update x64 += x (kernels_gmres.cu).
@@ -188,12 +189,21 @@ void launch_gmres_update_outer(const Grid& g, const float2* x, const GmresBufs& 
 template <class T> void gmres_smooth(const Grid& g, const OpView<T>& op, cx<T>* x, const cx<T>* b, int nu, int B,
                                      const int* active, const GmresBufs& gb, cudaStream_t s);
 
-// The same smoother on the fine level (kind 1) in four row-marching passes
+// The same smoother on the fine level (kind 1), complex128, in four row-marching passes
 // plus the update (gmres_march.cu); the partial buffer must hold
 // gmres_march_blocks() records per RHS.
-long long gmres_march_blocks(const Grid& g, bool fp64, int B);
+long long gmres_march_blocks(const Grid& g, int B);
 template <class T> void gmres_smooth_march(const Grid& g, const OpView<T>& op, cx<T>* x, const cx<T>* b, int nu,
                                            int B, const int* active, const GmresBufs& gb, cudaStream_t s);
+
+// The same smoother on the fine level in complex64: two row marches per step
+// in s-step form (sstep_march.cu).  x' alternates between x and xt; returns
+// the one that holds the result (with gb.outer the last step's result went to
+// the FP64 iterate instead).  The partial buffer must hold ss_march_blocks()
+// records per RHS.
+long long ss_march_blocks(const Grid& g, int B);
+float2* gmres_smooth_ss_march(const Grid& g, const OpView<float>& op, float2* x, float2* xt, const float2* b, int nu,
+                              int B, const int* active, const GmresBufs& gb, cudaStream_t s);
 
 // The same smoother on a Kronecker-form level (kinds 4, 5) with the kernels
 // that apply A written as column marches (kron_march.cu); the partial buffer

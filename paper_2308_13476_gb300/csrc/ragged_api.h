@@ -14,14 +14,17 @@ template <class T> struct RagLevel {
   Grid g;            // the problem's grid at this level (one right-hand side)
   OpView<T> op;      // its operator at this level
   cx<T>* x;          // iterate
+  cx<T>* xt;         // its alternate (complex64 fine level)
   const cx<T>* b;    // right-hand side
   GmresBufs gb;      // GMRES(3) vectors, scalars, reduction partials and ticket
   const int* active; // the problem's convergence mask
 };
 
-// nu GMRES(3) smoothing steps of the fine level (row marches), of a
-// Kronecker-form level (column marches); the update and the closing
-// Arnoldi pass shared by both.
+// nu GMRES(3) smoothing steps of the fine level (row marches; complex64 in
+// s-step form, which swaps x and xt in v at every step), of a Kronecker-form
+// level (column marches); the update and the closing Arnoldi pass shared by
+// both.
+void gmres_smooth_ss_march_rag(std::vector<RagLevel<float>>& v, int nu, cudaStream_t s);
 template <class T> void gmres_smooth_march_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream_t s,
                                                cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 template <class T> void gmres_smooth_kron_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream_t s);

@@ -53,14 +53,17 @@ __device__ __forceinline__ void ss_gram_add(T (&g)[SS_NV], cx<T> v0, cx<T> v1, c
 // the basis there (the remaining coefficients are 0), as a breakdown of the
 // Arnoldi process would.
 template <class V, class St> __device__ __forceinline__ void ss_solve(const V* g, float scale, float sigma, St* y) {
+  // the sums relative to |r|^2: z does not depend on their common factor, and
+  // near convergence |r|^2 alone is too small for products of its inverses
   float d[4], er[4][4], ei[4][4];   // <v_i, v_j> for i < j
+  const V f = V(1) / (g[0] > V(1e-36f) ? g[0] : V(1e-36f));
 #pragma unroll
   for (int i = 0, k = 4; i < 4; ++i) {
-    d[i] = (float)g[i];
+    d[i] = (float)(g[i] * f);
 #pragma unroll
     for (int j = i + 1; j < 4; ++j, k += 2) {
-      er[i][j] = (float)g[k];
-      ei[i][j] = (float)g[k + 1];
+      er[i][j] = (float)(g[k] * f);
+      ei[i][j] = (float)(g[k + 1] * f);
     }
   }
   // M_ij = <w_i, w_j> (lower triangle, i >= j) and f_i = <w_i, r>
@@ -118,6 +121,61 @@ template <class V, class St> __device__ __forceinline__ void ss_solve(const V* g
   y[3] = (St)(scale * s[1] * z1i);
   y[4] = (St)(scale * s[2] * z2r);
   y[5] = (St)(scale * s[2] * z2i);
+}
+
+// Grid-wide Gram sum of one right-hand side inside the kernel that forms v_3,
+// and the solve: every block of NT threads publishes its sums (float within
+// the warps, FP64 across them), the block with the last ticket adds the nrec
+// records (16 values side by side: thread t takes value t mod 16 of every
+// NT / 16-th record, in record order) and solves for y in the state S.
+// Reproducible: the order does not depend on which block is last.  Must be
+// reached by every thread of every block of the right-hand side.
+template <int NT>
+__device__ __forceinline__ void ss_finish(float (&g)[SS_NV], double* sh /* [NT] */, double* partial, unsigned* tickets,
+                                          int rhs, int nrec, int blk, int tid, float scale, float sigma, float* S) {
+  static_assert(NT % 32 == 0 && NT >= 32 && (SS_NV * (NT / 32)) <= NT && SS_NV == 16, "block shape");
+  __shared__ int s_last;
+  constexpr int W = NT / 32, G = NT / SS_NV;
+  const int lane = tid & 31, warp = tid >> 5;
+  const float t = lane_sum<SS_NV, float>(g, lane);
+  if ((lane & 1) == 0) sh[lane_value<SS_NV>(lane) * W + warp] = (double)t;
+  __syncthreads();
+  double* rec = partial + (long long)rhs * nrec * SS_NV;
+  if (tid < SS_NV) {
+    double v = sh[tid * W];
+#pragma unroll
+    for (int w = 1; w < W; ++w) v += sh[tid * W + w];
+    rec[blk * SS_NV + tid] = v;
+    __threadfence();
+  }
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&tickets[rhs], 1u) == (unsigned)(nrec - 1);
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  {
+    const double* q = rec + tid;   // record tid / 16, value tid % 16
+    double v = 0.0;
+    int b = tid / SS_NV;
+    for (; b + 3 * G < nrec; b += 4 * G, q += 4 * NT) {
+      const double a0 = __ldcg(q), a1 = __ldcg(q + NT), a2 = __ldcg(q + 2 * NT), a3 = __ldcg(q + 3 * NT);
+      v += (a0 + a1) + (a2 + a3);
+    }
+    for (; b < nrec; b += G, q += NT) v += __ldcg(q);
+    sh[tid] = v;
+  }
+  __syncthreads();
+  if (tid < SS_NV) {
+    double v = sh[tid];
+#pragma unroll
+    for (int k = 1; k < G; ++k) v += sh[k * SS_NV + tid];
+    sh[tid] = v;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    tickets[rhs] = 0u;
+    ss_solve(sh, scale, sigma, S);
+  }
 }
 
 }  // namespace hmg
