@@ -248,7 +248,7 @@ template <class T> static std::vector<LevelVec<T>>& vecs(mg_ctx* c);
 template <> std::vector<LevelVec<double>>& vecs<double>(mg_ctx* c) { return c->v64; }
 template <> std::vector<LevelVec<float>>& vecs<float>(mg_ctx* c) { return c->v32; }
 
-template <class T> static cudaError_t alloc_vectors(mg_ctx* c, LevelVec<T>& v, const Grid& g, bool gmres, bool kron) {
+template <class T> static cudaError_t alloc_vectors(mg_ctx* c, LevelVec<T>& v, const Grid& g, bool gmres) {
   const size_t bytes = sizeof(cx<T>) * (size_t)g.vstride * c->B;
   cudaError_t e;
   if ((e = dalloc(c, (void**)&v.x, bytes))) return e;
@@ -259,7 +259,6 @@ template <class T> static cudaError_t alloc_vectors(mg_ctx* c, LevelVec<T>& v, c
     for (int q = 0; q < 3; ++q)
       if ((e = dalloc(c, &v.gb.u[q], bytes))) return e;
     if ((e = dalloc(c, &v.gb.w, bytes))) return e;
-    if (kron && sizeof(T) == 4 && (e = dalloc(c, &v.gb.w2, bytes))) return e;   // fused column marches' second w
     v.gb.partial = c->partial;
     v.gb.tickets = c->tickets;
     v.gb.st = c->gst;
@@ -294,10 +293,17 @@ static bool use_ss_march(const mg_ctx* c, int l) {
   return c->opt.precision > 0 && c->opt.fuse && c->opt.march != 0 && c->lev[l].kind == 1;
 }
 
-// Returns the vector that holds the smoothed iterate: x, or xt.
+// Whether level l's pre-smoothing leaves the residual that the restriction
+// reads: complex64 GMRES(3) on the levels that store their Krylov vectors.
+static bool leaves_residual(const mg_ctx* c, int l) {
+  return c->opt.precision > 0 && c->opt.smoother == 1 && c->opt.fuse && c->opt.nu_pre > 0 && !use_ss_march(c, l);
+}
+
+// Returns the vector that holds the smoothed iterate: x, or xt.  want_r: leave
+// its residual in gb.u[0] (leaves_residual).
 template <class T>
 static cx<T>* gmres_level(mg_ctx* c, int l, cx<T>* x, cx<T>* xt, const cx<T>* b, int nu, const int* active,
-                          cudaStream_t s, double2* outer = nullptr, bool x_zero = false) {
+                          cudaStream_t s, double2* outer = nullptr, bool x_zero = false, bool want_r = false) {
   const Grid& g = c->lev[l].g;
   const OpView<T> op = opT<T>(c, l);
   GmresBufs gb = vecs<T>(c)[l].gb;
@@ -311,14 +317,12 @@ static cx<T>* gmres_level(mg_ctx* c, int l, cx<T>* x, cx<T>* xt, const cx<T>* b,
   gb.sigma = (float)ss_sigma(op.kind);
   if constexpr (sizeof(T) == 4) {
     if (use_ss_march(c, l)) return gmres_smooth_ss_march(g, op, x, xt, b, nu, c->B, active, gb, s);
-  }
-  const bool m = use_march(c, l);
-  if (m && op.kind >= 4) gmres_smooth_kron<T>(g, op, x, b, nu, c->B, active, gb, s);
-  else if constexpr (sizeof(T) == 8) {
-    if (m && op.kind == 1) gmres_smooth_march<T>(g, op, x, b, nu, c->B, active, gb, s);
-    else gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
+    gmres_smooth_ss(g, op, use_march(c, l), x, b, nu, want_r, c->B, active, gb, s);
   } else {
-    gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
+    const bool m = use_march(c, l);
+    if (m && op.kind >= 4) gmres_smooth_kron<T>(g, op, x, b, nu, c->B, active, gb, s);
+    else if (m && op.kind == 1) gmres_smooth_march<T>(g, op, x, b, nu, c->B, active, gb, s);
+    else gmres_smooth<T>(g, op, x, b, nu, c->B, active, gb, s);
   }
   return x;
 }
@@ -337,7 +341,7 @@ template <class T> struct Emit {
   // first GMRES(3) step then takes u0 = b without applying A
   std::vector<char> zx;
 
-  void smooth(int l, int nu, double2* outer = nullptr) {
+  void smooth(int l, int nu, double2* outer = nullptr, bool want_r = false) {
     const bool z = zx[l] != 0;
     zx[l] = 0;
     if (nu <= 0) return;
@@ -356,7 +360,7 @@ template <class T> struct Emit {
         std::swap(cur[l], oth[l]);
       }
     } else {
-      if (gmres_level<T>(c, l, cur[l], oth[l], V.b, nu, c->active, s, outer, z) != cur[l]) std::swap(cur[l], oth[l]);
+      if (gmres_level<T>(c, l, cur[l], oth[l], V.b, nu, c->active, s, outer, z, want_r) != cur[l]) std::swap(cur[l], oth[l]);
     }
   }
 
@@ -382,8 +386,11 @@ template <class T> struct Emit {
     auto& V = vecs<T>(c);
     const Grid& g = c->lev[l].g;
     const Grid& gc = c->lev[l + 1].g;
-    smooth(l, c->opt.nu_pre);
-    if (c->opt.fuse && c->lev[l].kind >= 4 && use_march(c, l)) {
+    const bool left = leaves_residual(c, l);
+    smooth(l, c->opt.nu_pre, nullptr, left);
+    if (left) {
+      launch_restrict<T>(g, gc, (const cx<T>*)V[l].gb.u[0], V[l + 1].b, c->B, c->active, c->xw, s);
+    } else if (c->opt.fuse && c->lev[l].kind >= 4 && use_march(c, l)) {
       // a Kronecker-form level: the residual as a column march (about a
       // twelfth of OpK::apply's arithmetic), then the restriction
       launch_kron_residual<T>(g, opT<T>(c, l), cur[l], V[l].b, V[l].r, c->B, c->active, c->opt.kron_chunk, s);
@@ -782,7 +789,7 @@ template <class T> struct EmitR {
     return (l == 0 && swapped && q(p)->lc > 0) != other ? V.t : V.x;
   }
 
-  void smooth(int l, const std::vector<int>& G, int nu) {
+  void smooth(int l, const std::vector<int>& G, int nu, bool want_r = false) {
     if (nu <= 0 || G.empty()) return;
     std::vector<RagLevel<T>> v;
     for (int p : G) {
@@ -797,16 +804,14 @@ template <class T> struct EmitR {
       if (l == 0) {
         gmres_smooth_ss_march_rag(v, nu, s);
         swapped ^= (nu & 1) != 0;
-        return;
+      } else {
+        gmres_smooth_ss_rag(v, nu, want_r, s);
       }
     }
     if constexpr (sizeof(T) == 8) {
-      if (l == 0) {
-        gmres_smooth_march_rag<T>(v, nu, s, c->side, c->ev_fork, c->ev_join);
-        return;
-      }
+      if (l == 0) gmres_smooth_march_rag<T>(v, nu, s, c->side, c->ev_fork, c->ev_join);
+      else gmres_smooth_kron_rag<T>(v, nu, s);
     }
- gmres_smooth_kron_rag<T>(v, nu, s);
   }
 
   // visit: the index among the level's visits from the level above
@@ -836,7 +841,8 @@ template <class T> struct EmitR {
         if (on) cudaStreamWaitEvent(s, c->cjoin[l], 0);
       }
     } join{c, s, l, !I.empty()};
-    smooth(l, G, c->opt.nu_pre);
+    const bool left = leaves_residual(q(G[0]), l);   // the same kernels for every problem of a flattened batch
+    smooth(l, G, c->opt.nu_pre, left);
     std::vector<RagXfer<T>> xf;
     std::vector<RagVec> zv;
     for (int p : G) {
@@ -846,7 +852,15 @@ template <class T> struct EmitR {
                               h->active});
       zv.push_back(RagVec{h->lev[l + 1].g, cur(p, l + 1), h->active});
     }
-    launch_resid_restrict_rag<T>(xf, c->sub[0]->xw, s);
+    if (left) {
+      if constexpr (sizeof(T) == 4) {
+        auto rf = xf;
+        for (size_t k = 0; k < G.size(); ++k) rf[k].x = (const cx<T>*)vecs<T>(q(G[k]))[l].gb.u[0];
+        launch_restrict_rag<T>(rf, c->sub[0]->xw, s);
+      }
+    } else {
+      launch_resid_restrict_rag<T>(xf, c->sub[0]->xw, s);
+    }
     launch_zero_rag<T>(zv, s);
     for (int g = 0; g < c->opt.cycle; ++g) cycle(l + 1, G, g);
     for (size_t k = 0; k < G.size(); ++k) xf[k].rc = cur(G[k], l + 1);   // the coarse correction
@@ -1112,7 +1126,7 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
   // work arrays
   long long nblk_max = 0;   // reduction partials: the most blocks of any level
   for (int l = 0; l < c->nlev; ++l) {
-    nblk_max = std::max(nblk_max, node_blocks(c->lev[l].g));
+    nblk_max = std::max({nblk_max, node_blocks(c->lev[l].g), mixed && gm ? sl_blocks(c->lev[l].g) : 0LL});
     if (c->lev[l].kind == 1)
       nblk_max = std::max({nblk_max, gmres_march_blocks(c->lev[l].g, c->B),
                            mixed && gm ? ss_march_blocks(c->lev[l].g, c->B) : 0LL});
@@ -1134,7 +1148,7 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
   // vectors
   if (!mixed) {
     c->v64.resize(c->nlev);
-    for (int l = 0; l < c->nlev; ++l) CK(alloc_vectors<double>(c, c->v64[l], c->lev[l].g, gm, c->lev[l].kind >= 4));
+    for (int l = 0; l < c->nlev; ++l) CK(alloc_vectors<double>(c, c->v64[l], c->lev[l].g, gm));
   } else {
     c->v64.resize(1);
     const size_t bytes = sizeof(double2) * (size_t)g0.vstride * c->B;
@@ -1142,7 +1156,7 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
     CK(dalloc(c, (void**)&c->v64[0].b, bytes));
     c->v32.resize(c->nlev);
     for (int l = 0; l < c->nlev; ++l) {
-      CK(alloc_vectors<float>(c, c->v32[l], c->lev[l].g, gm, c->lev[l].kind >= 4));
+      CK(alloc_vectors<float>(c, c->v32[l], c->lev[l].g, gm));
       if (l > 0 && c->lev[l].kind <= 3) {
         const Level& L = c->lev[l];
         const long long S = (long long)(2 * L.radius + 1) * (2 * L.radius + 1);

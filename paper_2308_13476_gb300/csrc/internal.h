@@ -165,7 +165,6 @@ void launch_export_stencil(const OpView<double>& op, int nx, int ny, int r, doub
 struct GmresBufs {
   void* u[3];          // Arnoldi vectors (unnormalised), precision T
   void* w;             // A v_j
-  void* w2;            // second w of the fused Kronecker-level marches (null: unfused)
   double* partial;     // block partials of the fused reductions
   unsigned* tickets;   // one per RHS, 0 at rest
   double* st;          // per-RHS scalars, see kernels_gmres.cu
@@ -182,10 +181,6 @@ struct GmresBufs {
                        // in every pass) and only sums |b|^2 for its norm
   float scale, sigma;  // complex64 s-step basis of the level (sstep.cuh)
 };
-// The last GMRES(3) update of a complex64 level-0 smoothing fused with the
-// FP64 refinement update x64 += x (kernels_gmres.cu).
-void launch_gmres_update_outer(const Grid& g, const float2* x, const GmresBufs& gb, int B, const int* active,
-                               cudaStream_t s);
 template <class T> void gmres_smooth(const Grid& g, const OpView<T>& op, cx<T>* x, const cx<T>* b, int nu, int B,
                                      const int* active, const GmresBufs& gb, cudaStream_t s);
 
@@ -205,8 +200,17 @@ long long ss_march_blocks(const Grid& g, int B);
 float2* gmres_smooth_ss_march(const Grid& g, const OpView<float>& op, float2* x, float2* xt, const float2* b, int nu,
                               int B, const int* active, const GmresBufs& gb, cudaStream_t s);
 
-// The same smoother on a Kronecker-form level (kinds 4, 5) with the kernels
-// that apply A written as column marches (kron_march.cu); the partial buffer
+// The same smoother in complex64 on a level that stores its Krylov vectors, in
+// s-step form (sstep_level.cu): Kronecker-form levels as column marches when
+// march, all others node-parallel.  want_r: leave r = b - A x in gb.u[0] (not
+// with gb.outer).  The partial buffer must hold sl_blocks() and
+// kron_march_blocks() records per RHS.
+long long sl_blocks(const Grid& g);
+void gmres_smooth_ss(const Grid& g, const OpView<float>& op, bool march, float2* x, const float2* b, int nu,
+                     bool want_r, int B, const int* active, const GmresBufs& gb, cudaStream_t s);
+
+// The same smoother on a Kronecker-form level (kinds 4, 5), complex128, with
+// the kernels that apply A written as column marches (kron_march.cu); the partial buffer
 // must hold kron_march_blocks() records per RHS.
 long long kron_march_blocks(const Grid& g, int B);
 template <class T> void gmres_smooth_kron(const Grid& g, const OpView<T>& op, cx<T>* x, const cx<T>* b, int nu, int B,

@@ -123,12 +123,9 @@ __global__ void __launch_bounds__(BX * BY) g_arn_a(Grid g, Op op, const cx<T>* _
   T* S = gstate<T>(st, rhs);
   if (S[G_BRK] != 0 || S[G_M] < J) return;   // block-uniform
   const cx<T>* uJ = J == 0 ? u0 : (J == 1 ? u1 : u2);
-  // complex64, J = 2: |w|^2 as well, for the Gram form of u3's norm
-  // (fin_b2_gram); w is then not stored (no g_arn_b<2> pass reads it)
-  constexpr int NG = (sizeof(T) == 4 && J == 2) ? 1 : 0;
-  T acc[2 * (J + 1) + NG];
+  T acc[2 * (J + 1)];
 #pragma unroll
-  for (int k = 0; k < 2 * (J + 1) + NG; ++k) acc[k] = T(0);
+  for (int k = 0; k < 2 * (J + 1); ++k) acc[k] = T(0);
   if (nv > 0) {
     const T sJ = (T)S[G_S + J];
     const cx<T>* us[3] = {u0, u1, u2};
@@ -138,13 +135,7 @@ __global__ void __launch_bounds__(BX * BY) g_arn_a(Grid g, Op op, const cx<T>* _
       Pack<T> a = apply_pack<T>(op, uJ + off, p, g.pitch, i0, j);
 #pragma unroll
       for (int n = 0; n < NP; ++n) a.v[n] = scl<T>(sJ, a.v[n]);
-      if constexpr (NG == 1) {
-#pragma unroll
-        for (int n = 0; n < NP; ++n)
-          if (n < nv) acc[2 * (J + 1)] += abs2<T>(a.v[n]);
-      } else {
-        store_pack(w + off, p, a, nv);
-      }
+      store_pack(w + off, p, a, nv);
 #pragma unroll
       for (int l = 0; l <= J; ++l) {
         const Pack<T> ul = load_pack(us[l] + off, p);
@@ -159,11 +150,10 @@ __global__ void __launch_bounds__(BX * BY) g_arn_a(Grid g, Op op, const cx<T>* _
       }
     }
   }
-  double v[2 * (J + 1) + NG];
-  if (reduce_last<2 * (J + 1) + NG, T>(acc, v, sh, partial, tickets, rhs, nblk, blk))
+  double v[2 * (J + 1)];
+  if (reduce_last<2 * (J + 1), T>(acc, v, sh, partial, tickets, rhs, nblk, blk))
     staged<T>(S, v, [](auto* s, const double* q) {
       fin_a<J, T>(s, q);
-      if constexpr (NG == 1) fin_b2_gram<T>(s, q[2 * (J + 1)]);
     });
 }
 
@@ -287,58 +277,6 @@ __global__ void __launch_bounds__(BX * BY) g_update(Grid g, cx<T>* __restrict__ 
   g_update_body<T>(blockIdx, gridDim, g, x, u0, u1, u2, st, active);
 }
 
-// The last GMRES(3) update of the level-0 post-smoothing of a complex64
-// cycle inside the FP64 refinement, fused with the refinement's update: the
-// updated complex64 iterate is the cycle's correction e, added to the FP64
-// iterate at once (x64 += e, the widening on the integer pipe) instead of
-// being stored and read back by a separate pass.  The complex64 iterate is
-// not stored (the next cycle starts from zero).  With no Arnoldi column
-// (m = 0) e is the iterate as it stands.
-__global__ void __launch_bounds__(BX * BY) g_update_outer(Grid g, const float2* __restrict__ x,
-                                                          const float2* __restrict__ u0, const float2* __restrict__ u1,
-                                                          const float2* __restrict__ u2, const double* __restrict__ st,
-                                                          double2* __restrict__ x64, const int* __restrict__ active) {
-  using T = float;
-  constexpr int NP = PK<T>::NP;
-  const int rhs = blockIdx.z;
-  const int i0 = (blockIdx.x * BX + threadIdx.x) * NP;
-  const int nv = min(NP, g.nx + 1 - i0);
-  const long long off = (long long)rhs * g.vstride;
-  if (active && !active[rhs]) return;
-  if (nv <= 0) return;
-  const T* S = gstate<T>(st, rhs);
-  const int m = (int)S[G_M];
-  const cx<T>* us[3] = {u0, u1, u2};
-  cx<T> c[3];
-#pragma unroll
-  for (int l = 0; l < 3; ++l) {
-    const T sl = S[G_S + l];
-    c[l] = mk<T>((T)(S[G_Y + 2 * l] * sl), (T)(S[G_Y + 2 * l + 1] * sl));
-  }
-  GROWS {
-    if (j > g.ny) break;
-    const int p = g.at(i0, j);
-    Pack<T> a = load_pack(x + off, p);
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      if (l < m) {
-        const Pack<T> ul = load_pack(us[l] + off, p);
-#pragma unroll
-        for (int n = 0; n < NP; ++n) a.v[n] = fma_c<T>(c[l], ul.v[n], a.v[n]);
-      }
-    }
-#pragma unroll
-    for (int n = 0; n < NP; ++n) {
-      if (n < nv) {
-        double2 xv = x64[off + p + n];
-        xv.x += f64_from_f32(a.v[n].x);
-        xv.y += f64_from_f32(a.v[n].y);
-        x64[off + p + n] = xv;
-      }
-    }
-  }
-}
-
 template <class T>
 __global__ void __launch_bounds__(BX * BY) g_update_rag(const __grid_constant__ RagLaunch<GuA<T>> L) {
   uint3 vb;
@@ -372,16 +310,9 @@ void gmres_smooth(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<T>* b,
       g_arn_a<T, Op, 1><<<grd, blk, 0, s>>>(g, op, v0, u1, u2, w, st, P, tk, active);
       g_arn_b<T, 1><<<grd, blk, 0, s>>>(g, v0, u1, u2, u2, w, st, P, tk, active, -1);
       g_arn_a<T, Op, 2><<<grd, blk, 0, s>>>(g, op, v0, u1, u2, w, st, P, tk, active);
-      if constexpr (sizeof(T) == 8)   // complex64: u3's norm came from the Gram form in g_arn_a<2>
-        g_arn_b<T, 2><<<grd, blk, 0, s>>>(g, v0, u1, u2, nullptr, w, st, P, tk, active, -1);
+      g_arn_b<T, 2><<<grd, blk, 0, s>>>(g, v0, u1, u2, nullptr, w, st, P, tk, active, -1);
       GmresBufs gs = gb;
       gs.u[0] = (void*)v0;
-      if constexpr (sizeof(T) == 4) {
-        if (step == nu - 1 && gb.outer) {
-          launch_gmres_update_outer(g, x, gs, B, active, s);
-          continue;
-        }
-      }
       g_update<T><<<grd, blk, 0, s>>>(g, x, v0, u1, u2, st, active);
     }
   });
@@ -393,13 +324,6 @@ void launch_gmres_update(const Grid& g, cx<T>* x, const GmresBufs& gb, int B, co
   dim3 grd(cdiv(g.nx + 1, BX * PK<T>::NP), cdiv(g.ny + 1, BY * g.ry), B);
   g_update<T><<<grd, dim3(BX, BY), 0, s>>>(g, x, (const cx<T>*)gb.u[0], (const cx<T>*)gb.u[1],
                                           (const cx<T>*)gb.u[2], gb.st, active);
-}
-
-void launch_gmres_update_outer(const Grid& g, const float2* x, const GmresBufs& gb, int B, const int* active,
-                               cudaStream_t s) {
-  dim3 grd(cdiv(g.nx + 1, BX * PK<float>::NP), cdiv(g.ny + 1, BY * g.ry), B);
-  g_update_outer<<<grd, dim3(BX, BY), 0, s>>>(g, x, (const float2*)gb.u[0], (const float2*)gb.u[1],
-                                              (const float2*)gb.u[2], gb.st, gb.outer, active);
 }
 
 template <class T, int J>
@@ -433,24 +357,14 @@ void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next, int ws, c
 }
 
 template void launch_gmres_update_rag<double>(const std::vector<RagLevel<double>>&, cudaStream_t);
-template void launch_gmres_update_rag<float>(const std::vector<RagLevel<float>>&, cudaStream_t);
 template void launch_arn_b_rag<double, 0>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
 template void launch_arn_b_rag<double, 1>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
 template void launch_arn_b_rag<double, 2>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
-template void launch_arn_b_rag<float, 0>(const std::vector<RagLevel<float>>&, bool, int, cudaStream_t);
-template void launch_arn_b_rag<float, 1>(const std::vector<RagLevel<float>>&, bool, int, cudaStream_t);
-template void launch_arn_b_rag<float, 2>(const std::vector<RagLevel<float>>&, bool, int, cudaStream_t);
 template void launch_arn_b<double, 0>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
 template void launch_arn_b<double, 1>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
 template void launch_arn_b<double, 2>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
-template void launch_arn_b<float, 0>(const Grid&, const GmresBufs&, float2*, int, const int*, cudaStream_t, int);
-template void launch_arn_b<float, 1>(const Grid&, const GmresBufs&, float2*, int, const int*, cudaStream_t, int);
-template void launch_arn_b<float, 2>(const Grid&, const GmresBufs&, float2*, int, const int*, cudaStream_t, int);
 template void launch_gmres_update<double>(const Grid&, double2*, const GmresBufs&, int, const int*, cudaStream_t);
-template void launch_gmres_update<float>(const Grid&, float2*, const GmresBufs&, int, const int*, cudaStream_t);
 template void gmres_smooth<double>(const Grid&, const OpView<double>&, double2*, const double2*, int, int, const int*,
                                    const GmresBufs&, cudaStream_t);
-template void gmres_smooth<float>(const Grid&, const OpView<float>&, float2*, const float2*, int, int, const int*,
-                                  const GmresBufs&, cudaStream_t);
 
 }  // namespace hmg

@@ -296,9 +296,11 @@ __global__ void __launch_bounds__(BX * BY) k_vecnorm_fin(Grid g, const cx<T>* __
 
 // r_c(I,J) = 1/4 sum_{a,b=-2..2} w(a) w(b) r_f(2I+a, 2J+b)   (R = P^T / 4)
 template <class T>
-__global__ void __launch_bounds__(BX * BY) k_restrict(Grid gf, Grid g, const cx<T>* __restrict__ rf,
-                                                      cx<T>* __restrict__ rc, const int* __restrict__ active,
-                                                      Xfer xw) {
+__device__ __forceinline__ void k_restrict_body(uint3 vblk, dim3 vgrid, Grid gf, Grid g, const cx<T>* __restrict__ rf,
+                                                cx<T>* __restrict__ rc, const int* __restrict__ active, Xfer xw) {
+  const uint3 blockIdx = vblk;   // the block and grid inside this problem's launch
+  const dim3 gridDim = vgrid;
+  (void)gridDim;
   NODE_INDEX
   const T c0 = T(xw.w0), c1 = T(xw.w1), c2 = T(xw.w2);
   if (active && !active[rhs]) return;
@@ -318,6 +320,31 @@ __global__ void __launch_bounds__(BX * BY) k_restrict(Grid gf, Grid g, const cx<
     }
     rc[off + g.at(i, j)] = scl<T>(T(0.25), acc);
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(BX * BY) k_restrict(Grid gf, Grid g, const cx<T>* __restrict__ rf,
+                                                      cx<T>* __restrict__ rc, const int* __restrict__ active,
+                                                      Xfer xw) {
+  k_restrict_body<T>(blockIdx, gridDim, gf, g, rf, rc, active, xw);
+}
+
+// Arguments of the flattened restriction.
+template <class T>
+struct ReA {
+  Grid gf;
+  Grid gc;
+  const cx<T>* rf;
+  cx<T>* rc;
+  const int* active;
+  Xfer xw;
+};
+template <class T>
+__global__ void __launch_bounds__(BX * BY) k_restrict_rag(const __grid_constant__ RagLaunch<ReA<T>> L) {
+  uint3 vb;
+  dim3 vg;
+  const ReA<T>& a = L.a[rag_problem(L, blockIdx.x, vb, vg)];
+  k_restrict_body<T>(vb, vg, a.gf, a.gc, a.rf, a.rc, a.active, a.xw);
 }
 
 // x_f(i,j) += sum_{I,J} P(i,I) P(j,J) e_c(I,J)   (Eq. (xex) in each direction)
@@ -524,6 +551,18 @@ template <class T> void launch_zero_rag(const std::vector<RagVec>& v, cudaStream
 }
 template void launch_zero_rag<double>(const std::vector<RagVec>&, cudaStream_t);
 template void launch_zero_rag<float>(const std::vector<RagVec>&, cudaStream_t);
+
+template <class T> void launch_restrict_rag(const std::vector<RagXfer<T>>& v, const Xfer& xw, cudaStream_t s) {
+  rag_launch<ReA<T>>((int)v.size(), k_restrict_rag<T>, dim3(BX, BY), 0, s, [&](int q, ReA<T>& a, int& gx, int& gy) {
+    const RagXfer<T>& X = v[q];
+    a = ReA<T>{X.gf, X.gc, X.x, X.rc, X.active, xw};
+    const dim3 d = node_grid(X.gc, 1);
+    gx = (int)d.x;
+    gy = (int)d.y;
+    return true;
+  });
+}
+template void launch_restrict_rag<float>(const std::vector<RagXfer<float>>&, const Xfer&, cudaStream_t);
 
 template <class T> void launch_prolong_add_rag(const std::vector<RagXfer<T>>& v, const Xfer& xw, cudaStream_t s) {
   rag_launch<PaA<T>>((int)v.size(), k_prolong_add_rag<T>, dim3(BX, BY), 0, s, [&](int q, PaA<T>& a, int& gx, int& gy) {

@@ -25,6 +25,7 @@ template <class T> struct RagLevel {
 // level (column marches); the update and the closing Arnoldi pass shared by
 // both.
 void gmres_smooth_ss_march_rag(std::vector<RagLevel<float>>& v, int nu, cudaStream_t s);
+void gmres_smooth_ss_rag(const std::vector<RagLevel<float>>& v, int nu, bool want_r, cudaStream_t s);
 template <class T> void gmres_smooth_march_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream_t s,
                                                cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 template <class T> void gmres_smooth_kron_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream_t s);
@@ -44,6 +45,8 @@ template <class T> struct RagXfer {
   const int* active;
 };
 template <class T> void launch_resid_restrict_rag(const std::vector<RagXfer<T>>& v, const Xfer& xw, cudaStream_t s);
+// b_{l+1} = R r, the residual in x
+template <class T> void launch_restrict_rag(const std::vector<RagXfer<T>>& v, const Xfer& xw, cudaStream_t s);
 template <class T> void launch_prolong_add_rag(const std::vector<RagXfer<T>>& v, const Xfer& xw, cudaStream_t s);
 
 // Zero a vector of each problem (its grid with one right-hand side).
