@@ -28,70 +28,96 @@
 namespace hmg {
 
 namespace {
-constexpr int NA_BX = 32, NA_BY = 8, NA_RY = 4;      // a block covers 32 x 32 grid nodes
+constexpr int NA_TILE = 32;                           // grids are accepted by their count of 32 x 32 tiles
 constexpr int NA_MAX_BLOCKS = 16384;                  // -> at most 16.7 M nodes
+constexpr int NA_NT = 256;                            // threads per block
+constexpr int NA_RESIDENT = 152 * 6;                  // blocks of the one-node form that run at once
 constexpr int NA_MAX_DEVICES = 64;
 }  // namespace
 
 // [blk][2] partial sums (|r|^2, |b|^2) followed by the ticket; 256 KiB + 256 B.
 static __device__ __align__(256) double g_noalloc_scratch[2 * NA_MAX_BLOCKS + 32];
 
-// Same operator as Op0 (ghost-eliminated Sommerfeld rows scaled by 1/2 and
-// 1/4), on the caller's dense [ny+1][nx+1] layout, neighbours off the grid
-// read as zero.
-__global__ void __launch_bounds__(NA_BX * NA_BY)
-    k_resnorm_dense(int nx, int ny, double inv_h2, double inv_h, double kc, const double* __restrict__ kf,
-                    const double2* __restrict__ x, const double2* __restrict__ b, double* scratch,
-                    double* __restrict__ out) {
-  __shared__ double sh[2 * 32];
+// The norms on the caller's dense [ny+1][nx+1] layout, RY nodes per thread: a
+// block takes RY * 256 consecutive nodes, so that no thread is left without
+// one at the grid's right edge.
+//
+// What bounds it is the FP64 pipe (two multiply-adds per clock and SM), so an
+// interior node costs 14 FP64 instructions: b - d x + (1/h^2) (E + W + N + S)
+// with d = 4/h^2 - k^2, five per component, and two for each norm.  Edge rows
+// and columns take the operator of the solver (Op0::apply5) on zero off the
+// grid.  One node per thread while all blocks run at once: the pipe is then
+// evenly loaded and every load is in flight; above that four, for fewer
+// records in the last block.  Per call, 32 x 32-node tiles with 35 FP64
+// instructions per node -> this form: 257^2 18.7 -> 12.4 us (most of it the
+// launches of the clear and the kernel), 513^2 29 -> 20.6 us, 1001^2 82 -> 43
+// us, 2001^2 287 -> 136 us.
+template <int RY, bool VK>
+__global__ void __launch_bounds__(NA_NT) k_resnorm_dense(const __grid_constant__ Op0<double> op, int nodes, double dc,
+                                                         const double2* __restrict__ x, const double2* __restrict__ b,
+                                                         double* scratch, double* __restrict__ out) {
+  __shared__ double sh[2 * NA_NT / 32];
   __shared__ int s_last;
-  const int i = blockIdx.x * NA_BX + threadIdx.x;
-  const int nblk = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
+  const int nx = op.nx, ny = op.ny, n1 = nx + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nblk = gridDim.x, blk = blockIdx.x;
+  const double ih2 = op.c.inv_h2;
   double v[2] = {0.0, 0.0};
-  if (i <= nx) {
-    for (int r_ = 0, j = blockIdx.y * NA_BY * NA_RY + threadIdx.y; r_ < NA_RY; ++r_, j += NA_BY) {
-      if (j > ny) break;
-      const long long q = (long long)j * (nx + 1) + i;
-      const int bx = (i == 0 || i == nx), by = (j == 0 || j == ny);
-      const double wx = bx ? 0.5 : 1.0, wy = by ? 0.5 : 1.0, w = wx * wy;
-      const double k = kf ? kf[q] : kc;
-      const double2 xp = x[q];
-      const double2 z = make_double2(0.0, 0.0);
-      const double2 xe = i < nx ? x[q + 1] : z, xw = i > 0 ? x[q - 1] : z;
-      const double2 xn = j < ny ? x[q + nx + 1] : z, xs = j > 0 ? x[q - nx - 1] : z;
-      const double sr = wy * (xe.x + xw.x) + wx * (xn.x + xs.x), si = wy * (xe.y + xw.y) + wx * (xn.y + xs.y);
-      const double re = (4.0 * w * xp.x - sr) * inv_h2 - (w * (k * k)) * xp.x;
-      const double im = (4.0 * w * xp.y - si) * inv_h2 - (w * (k * k)) * xp.y;
-      const double sb = (k * inv_h) * (bx * wy + wx * by);
-      const double2 bq = b[q];
-      const double rx = bq.x - (re + sb * xp.y), ry = bq.y - (im - sb * xp.x);
-      v[0] += rx * rx + ry * ry;
-      v[1] += bq.x * bq.x + bq.y * bq.y;
+#pragma unroll
+  for (int r = 0; r < RY; ++r) {
+    const int q = (blk * RY + r) * NA_NT + tid;
+    if (q >= nodes) break;
+    const int j = q / n1, i = q - j * n1;
+    const double2 xp = x[q], bq = b[q], z = make_double2(0.0, 0.0);
+    const double2 xe = i < nx ? x[q + 1] : z, xw = i > 0 ? x[q - 1] : z;
+    const double2 xn = j < ny ? x[q + n1] : z, xs = j > 0 ? x[q - n1] : z;
+    double2 t;
+    if (i > 0 && i < nx && j > 0 && j < ny) {
+      double d = dc;
+      if constexpr (VK) {
+        const double k = op.kf[q];
+        d = fma(-k, k, 4.0 * ih2);
+      }
+      t.x = fma(ih2, (xe.x + xw.x) + (xn.x + xs.x), fma(-d, xp.x, bq.x));
+      t.y = fma(ih2, (xe.y + xw.y) + (xn.y + xs.y), fma(-d, xp.y, bq.y));
+    } else {
+      t = sub<double>(bq, op.apply5(xp, xe, xw, xn, xs, i, j));
     }
+    v[0] = fma(t.x, t.x, fma(t.y, t.y, v[0]));
+    v[1] = fma(bq.x, bq.x, fma(bq.y, bq.y, v[1]));
   }
-  block_sum<2>(v, sh);
-  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+  // both sums of the block in threads 0 and 16 (FP64 adds: 6 per warp, then one per warp)
+  auto block_sums = [&](double (&a)[2]) {
+    const double t = lane_sum<2, double>(a, lane);
+    if ((lane & 15) == 0) sh[lane_value<2>(lane) * (NA_NT / 32) + warp] = t;
+    __syncthreads();
+    double s = 0.0;
+    if (warp == 0 && (lane & 15) == 0) {
+#pragma unroll
+      for (int w = 0; w < NA_NT / 32; ++w) s += sh[lane_value<2>(lane) * (NA_NT / 32) + w];
+    }
+    return s;
+  };
+  const bool own = warp == 0 && (lane & 15) == 0;
+  const double s = block_sums(v);
   unsigned* ticket = reinterpret_cast<unsigned*>(scratch + 2 * NA_MAX_BLOCKS);
-  if (tid == 0) {
-    scratch[2 * blk] = v[0];
-    scratch[2 * blk + 1] = v[1];
+  if (own) {
+    scratch[2 * blk + lane_value<2>(lane)] = s;
     __threadfence();
-    s_last = atomicAdd(ticket, 1u) == (unsigned)(nblk - 1);
   }
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(ticket, 1u) == (unsigned)(nblk - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   double a[2] = {0.0, 0.0};
-  for (int q = tid; q < nblk; q += blockDim.x * blockDim.y) {
-    a[0] += __ldcg(scratch + 2 * q);
-    a[1] += __ldcg(scratch + 2 * q + 1);
+  for (int q = tid; q < nblk; q += NA_NT) {
+    const double2 p = __ldcg(reinterpret_cast<const double2*>(scratch) + q);
+    a[0] += p.x;
+    a[1] += p.y;
   }
-  block_sum<2>(a, sh);
-  if (tid == 0) {
-    out[0] = sqrt(a[0]);
-    out[1] = sqrt(a[1]);
-    *ticket = 0u;
-  }
+  const double total = block_sums(a);
+  if (own) out[lane_value<2>(lane)] = sqrt(total);
+  if (tid == 0) *ticket = 0u;
 }
 
 }  // namespace hmg
@@ -107,7 +133,7 @@ extern "C" mg_status mg_residual_norm_static(int nx, int ny, double h, const dou
     hmg_set_error("mg_residual_norm_static: need nx, ny >= 2, h > 0, k >= 0 and non-NULL x, b, out");
     return MG_EINVAL;
   }
-  const long long nbx = (nx + 1 + NA_BX - 1) / NA_BX, nby = (ny + 1 + NA_BY * NA_RY - 1) / (NA_BY * NA_RY);
+  const long long nbx = cdiv(nx + 1LL, NA_TILE), nby = cdiv(ny + 1LL, NA_TILE);
   if (nbx * nby > NA_MAX_BLOCKS) {
     hmg_set_error("mg_residual_norm_static: grid too large for the static scratch (at most 16384 blocks of 32 x 32 "
                   "nodes, about 16.7 M nodes)");
@@ -139,9 +165,19 @@ extern "C" mg_status mg_residual_norm_static(int nx, int ny, double h, const dou
     hmg_set_error("mg_residual_norm_static: clearing the ticket failed");
     return MG_ECUDA;
   }
-  k_resnorm_dense<<<dim3((unsigned)nbx, (unsigned)nby), dim3(NA_BX, NA_BY), 0, s>>>(
-      nx, ny, 1.0 / (h * h), 1.0 / h, k_field ? 0.0 : k_const, k_field, (const double2*)x, (const double2*)b, scratch,
-      out);
+  const int nodes = (nx + 1) * (ny + 1);   // at most 2^24 here
+  Op0<double> op{};
+  op.c.inv_h2 = 1.0 / (h * h);
+  op.c.inv_h = 1.0 / h;
+  op.c.k = k_field ? 0.0 : k_const;
+  op.kf = k_field;
+  op.nx = nx;
+  op.ny = ny;
+  const double dc = 4.0 * op.c.inv_h2 - op.c.k * op.c.k;
+  const double2 *xv = (const double2*)x, *bv = (const double2*)b;
+  auto launch = [&](auto kern, int ry) { kern<<<cdiv(nodes, NA_NT * ry), NA_NT, 0, s>>>(op, nodes, dc, xv, bv, scratch, out); };
+  if (cdiv(nodes, NA_NT) <= NA_RESIDENT) launch(k_field ? k_resnorm_dense<1, true> : k_resnorm_dense<1, false>, 1);
+  else launch(k_field ? k_resnorm_dense<4, true> : k_resnorm_dense<4, false>, 4);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     hmg_set_error("mg_residual_norm_static: kernel launch failed");
