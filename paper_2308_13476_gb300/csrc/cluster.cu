@@ -250,15 +250,25 @@ __device__ __forceinline__ cx<T> combine(const Blk<T>& B, const Slab<T>& s, int 
     return L.c0.abc2 ? Op0<T, true>{L.c0, L.kf, L.nx, L.ny}.apply5(X[0], xe, xw, xn, xs, i, j)
                      : Op0<T>{L.c0, L.kf, L.nx, L.ny}.apply5(X[0], xe, xw, xn, xs, i, j);
   } else {
+    // Stored stencil: the coefficients come from L2 at every application (a
+    // slab's do not fit on chip), so the loads are issued in groups of rows
+    // before the multiply-adds that wait for them (one load at a time was the
+    // chain that took 446 us of a layered 1281 x 449 cycle); a coupling off the
+    // grid has a stored coefficient, and its node value is taken as zero.
+    constexpr int K = 2 * R + 1, G = sizeof(T) == 8 ? 2 : R == 2 ? 5 : 4;
     cx<T> acc = mk<T>(0, 0);
     const cx<T>* st = L.st + (long long)j * n1 + i;
 #pragma unroll
-    for (int dy = -R; dy <= R; ++dy) {
-      if ((unsigned)(j + dy) > (unsigned)L.ny) continue;
+    for (int d0 = 0; d0 < K; d0 += G) {
+      cx<T> c[G * K];
 #pragma unroll
-      for (int dx = -R; dx <= R; ++dx)
-        if ((unsigned)(i + dx) < (unsigned)n1)
-          acc = fma_c<T>(st[((dy + R) * (2 * R + 1) + dx + R) * L.plane], X[dy * n1 + dx], acc);
+      for (int e = 0; e < G * K && d0 * K + e < K * K; ++e) c[e] = __ldg(st + (d0 * K + e) * L.plane);
+#pragma unroll
+      for (int e = 0; e < G * K && d0 * K + e < K * K; ++e) {
+        const int dy = d0 + e / K - R, dx = e % K - R;
+        if ((unsigned)(j + dy) <= (unsigned)L.ny && (unsigned)(i + dx) < (unsigned)n1)
+          acc = fma_c<T>(c[e], X[dy * n1 + dx], acc);
+      }
     }
     return acc;
   }

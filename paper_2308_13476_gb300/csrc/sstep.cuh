@@ -20,6 +20,7 @@
 // follow modified Gram-Schmidt to rounding.
 #pragma once
 #include "common.cuh"
+#include "gmres.cuh"
 
 namespace hmg {
 
@@ -123,59 +124,78 @@ template <class V, class St> __device__ __forceinline__ void ss_solve(const V* g
   y[5] = (St)(scale * s[2] * z2i);
 }
 
-// Grid-wide Gram sum of one right-hand side inside the kernel that forms v_3,
-// and the solve: every block of NT threads publishes its sums (float within
-// the warps, FP64 across them), the block with the last ticket adds the nrec
-// records (16 values side by side: thread t takes value t mod 16 of every
-// NT / 16-th record, in record order) and solves for y in the state S.
-// Reproducible: the order does not depend on which block is last.  Must be
-// reached by every thread of every block of the right-hand side.
-template <int NT>
-__device__ __forceinline__ void ss_finish(float (&g)[SS_NV], double* sh /* [NT] */, double* partial, unsigned* tickets,
-                                          int rhs, int nrec, int blk, int tid, float scale, float sigma, float* S) {
-  static_assert(NT % 32 == 0 && NT >= 32 && (SS_NV * (NT / 32)) <= NT && SS_NV == 16, "block shape");
-  __shared__ int s_last;
-  constexpr int W = NT / 32, G = NT / SS_NV;
-  const int lane = tid & 31, warp = tid >> 5;
+// The block's Gram sums of one right-hand side by warp, sh[value * warps +
+// warp]: float within the warps, FP64 from there on.
+template <int NT> __device__ __forceinline__ void ss_warp_sums(float (&g)[SS_NV], double* sh /* [SS_NV * NT / 32] */, int tid) {
+  const int lane = tid & 31;
   const float t = lane_sum<SS_NV, float>(g, lane);
-  if ((lane & 1) == 0) sh[lane_value<SS_NV>(lane) * W + warp] = (double)t;
+  if ((lane & 1) == 0) sh[lane_value<SS_NV>(lane) * (NT / 32) + (tid >> 5)] = (double)t;
+}
+
+// Grid-wide Gram sums of RB right-hand sides from rhs0 on inside the kernel
+// that forms v_3, and the solves: every block publishes its sums (sh:
+// ss_warp_sums of each right-hand side, one after the other), the block with
+// the last ticket adds the nrec records of each and solves for y in the state
+// at S.  The RB right-hand sides share the ticket, the fences and the wait for
+// the records: NT / RB threads take one of them, 16 values side by side,
+// every thread one value of every NT / RB / 16-th record, in record order.
+// act: bit q set if right-hand side rhs0 + q takes part.  Reproducible: the
+// order does not depend on which block is last.  Must be reached by every
+// thread of every block of these right-hand sides; the records of tickets[rhs0]
+// are complete at the last ticket.
+template <int NT, int RB>
+__device__ __forceinline__ void ss_finish_rb(double* sh /* [RB * SS_NV * max(NT / 32, NT / RB / 16)] */, double* partial,
+                                             unsigned* tickets, int rhs0, unsigned act, int nrec, int blk, int tid,
+                                             float scale, float sigma, double* st) {
+  constexpr int W = NT / 32, N = NT / RB, G = N / SS_NV;   // threads and records per pass of one right-hand side
+  static_assert(NT % 32 == 0 && SS_NV * RB <= NT && N % SS_NV == 0 && N % 32 == 0 && SS_NV == 16, "block shape");
+  __shared__ int s_last;
   __syncthreads();
-  double* rec = partial + (long long)rhs * nrec * SS_NV;
-  if (tid < SS_NV) {
+  if (tid < SS_NV * RB && (act >> (tid / SS_NV) & 1)) {
     double v = sh[tid * W];
 #pragma unroll
     for (int w = 1; w < W; ++w) v += sh[tid * W + w];
-    rec[blk * SS_NV + tid] = v;
+    partial[((long long)(rhs0 + tid / SS_NV) * nrec + blk) * SS_NV + tid % SS_NV] = v;
     __threadfence();
   }
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&tickets[rhs], 1u) == (unsigned)(nrec - 1);
+  if (tid == 0) s_last = atomicAdd(&tickets[rhs0], 1u) == (unsigned)(nrec - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  {
-    const double* q = rec + tid;   // record tid / 16, value tid % 16
+  const int q = tid / N, t = tid - q * N;
+  const bool on = act >> q & 1;
+  if (on) {
+    const double* rec = partial + (long long)(rhs0 + q) * nrec * SS_NV + t;   // record t / 16, value t % 16
     double v = 0.0;
-    int b = tid / SS_NV;
-    for (; b + 3 * G < nrec; b += 4 * G, q += 4 * NT) {
-      const double a0 = __ldcg(q), a1 = __ldcg(q + NT), a2 = __ldcg(q + 2 * NT), a3 = __ldcg(q + 3 * NT);
-      v += (a0 + a1) + (a2 + a3);
+    int b = t / SS_NV;
+    for (; b + 7 * G < nrec; b += 8 * G, rec += 8 * N) {
+      double a[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) a[k] = __ldcg(rec + k * N);
+      v += ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
     }
-    for (; b < nrec; b += G, q += NT) v += __ldcg(q);
+    for (; b < nrec; b += G, rec += N) v += __ldcg(rec);
     sh[tid] = v;
   }
   __syncthreads();
-  if (tid < SS_NV) {
+  if (on && t < SS_NV) {
     double v = sh[tid];
 #pragma unroll
-    for (int k = 1; k < G; ++k) v += sh[k * SS_NV + tid];
+    for (int k = 1; k < G; ++k) v += sh[tid + k * SS_NV];
     sh[tid] = v;
   }
   __syncthreads();
-  if (tid == 0) {
-    tickets[rhs] = 0u;
-    ss_solve(sh, scale, sigma, S);
-  }
+  if (tid == 0) tickets[rhs0] = 0u;
+  if (on && t == 0) ss_solve(sh + q * N, scale, sigma, gstate<float>(st, rhs0 + q));
+}
+
+// The same for one right-hand side (sh: [NT]).
+template <int NT>
+__device__ __forceinline__ void ss_finish(float (&g)[SS_NV], double* sh, double* partial, unsigned* tickets, int rhs,
+                                          int nrec, int blk, int tid, float scale, float sigma, double* st) {
+  ss_warp_sums<NT>(g, sh, tid);
+  ss_finish_rb<NT, 1>(sh, partial, tickets, rhs, 1u, nrec, blk, tid, scale, sigma, st);
 }
 
 }  // namespace hmg

@@ -115,13 +115,16 @@ __global__ void __launch_bounds__(BX * BY) sl_apply(const __grid_constant__ SlA 
   const int i0 = (blockIdx.x * BX + threadIdx.x) * 2, j = blockIdx.y * BY + threadIdx.y;
   const int nv = j <= g.ny ? min(2, g.nx + 1 - i0) : 0;
   const long long vs = g.vstride, off = r0 * vs;
-  const int p = g.at(i0, j);
+  const int p = g.at(i0, j), tid = threadIdx.x + threadIdx.y * BX;
+  constexpr int NT = BX * BY;
   Pack<float> y[RB];
   if (nv > 0) RbApply<Op, RB>::run(op, a.v + off, vs, nrb, p, g.pitch, i0, j, y);
-  __shared__ double sh[MODE == GRAM ? BX * BY : 1];
+  __shared__ double sh[MODE != GRAM ? 1 : RB == 1 ? NT : RB * SS_NV * (NT / 32)];
+  unsigned act = 0;   // block-uniform
 #pragma unroll
   for (int q = 0; q < RB; ++q) {
-    if (q >= nrb || (a.active && !a.active[r0 + q])) continue;   // block-uniform
+    if (q >= nrb || (a.active && !a.active[r0 + q])) continue;
+    act |= 1u << q;
     const long long o = off + q * vs;
     float gm[SS_NV];
     if constexpr (MODE == GRAM) {
@@ -147,12 +150,74 @@ __global__ void __launch_bounds__(BX * BY) sl_apply(const __grid_constant__ SlA 
       }
       if (MODE != GRAM || a.out) store_pack(a.out + o, p, w, nv);
     }
-    if constexpr (MODE == GRAM) {
-      ss_finish<BX * BY>(gm, sh, a.partial, a.tickets, r0 + q, gridDim.x * gridDim.y,
-                         blockIdx.y * gridDim.x + blockIdx.x, threadIdx.x + threadIdx.y * BX, a.scale, a.sigma,
-                         gstate<float>(a.st, r0 + q));
-      __syncthreads();   // the scratch is free again
+    if constexpr (MODE == GRAM) ss_warp_sums<NT>(gm, sh + q * SS_NV * (NT / 32), tid);
+  }
+  if constexpr (MODE == GRAM)
+    ss_finish_rb<NT, RB>(sh, a.partial, a.tickets, r0, act, gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x,
+                         tid, a.scale, a.sigma, a.st);
+}
+
+// One node per thread and one right-hand side per block, stored stencils: the
+// launch of a level that the blocks above would leave under-filled.  A
+// thread's (2R+1)^2 coefficients come from L2 once and nothing is reused, so
+// what bounds it is how many of those loads are in flight: they are issued in
+// groups of stencil rows (all five rows of radius 2, three of radius 3 at a
+// time), coefficients and v together, before the first multiply-add, and a
+// thread has half the loads and the launch twice the threads of the pair form.
+// Layered model 1281 x 449, one right-hand side, with the grouped loads of the
+// cluster launch (cluster.cu): 237 -> 162 ms.
+template <int R>
+__device__ __forceinline__ float2 stencil_node(const float2* st, long long plane, const float2* v, int pitch) {
+  constexpr int K = 2 * R + 1, G = R == 2 ? 5 : 3;
+  float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int d0 = 0; d0 < K; d0 += G) {
+    float2 c[G * K], x[G * K];
+#pragma unroll
+    for (int e = 0; e < G * K; ++e) {
+      if (d0 * K + e >= K * K) break;
+      c[e] = __ldg(st + (long long)(d0 * K + e) * plane);
+      x[e] = v[(d0 + e / K - R) * pitch + e % K - R];
     }
+#pragma unroll
+    for (int e = 0; e < G * K; ++e) {
+      if (d0 * K + e >= K * K) break;
+      acc = fma_c<float>(c[e], x[e], acc);
+    }
+  }
+  return acc;
+}
+
+template <int R, int MODE, int NY>
+__global__ void __launch_bounds__(BX * NY, 512 / (BX * NY)) sl_one(const __grid_constant__ SlA a,
+                                                                   const __grid_constant__ OpS<float, R> op) {
+  const Grid& g = a.g;
+  const int rhs = blockIdx.z;
+  if (a.active && !a.active[rhs]) return;
+  const int i = blockIdx.x * BX + threadIdx.x, j = blockIdx.y * NY + threadIdx.y;
+  const long long off = (long long)rhs * g.vstride;
+  float gm[SS_NV];
+  if constexpr (MODE == GRAM) {
+#pragma unroll
+    for (int k = 0; k < SS_NV; ++k) gm[k] = 0.f;
+  }
+  if (i <= g.nx && j <= g.ny) {
+    const long long p = off + g.at(i, j);
+    const float2 y = stencil_node<R>(op.st + (long long)j * (op.nx + 1) + i, op.plane, a.v + p, g.pitch);
+    float2 w;
+    if constexpr (MODE == RES) {
+      w = sub2(a.b[p], y);
+    } else {
+      const float2 v = a.v[p];
+      w = fma2(bc2(a.scale), y, mul2(bc2(-a.sigma), v));
+      if constexpr (MODE == GRAM) ss_gram_add(gm, a.r[p], a.v1[p], v, w);
+    }
+    if (MODE != GRAM || a.out) a.out[p] = w;
+  }
+  if constexpr (MODE == GRAM) {
+    __shared__ double sh[BX * NY];
+    ss_finish<BX * NY>(gm, sh, a.partial, a.tickets, rhs, gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x,
+                       threadIdx.x + threadIdx.y * BX, a.scale, a.sigma, a.st);
   }
 }
 
@@ -223,7 +288,7 @@ template <int R, int MODE> __device__ __forceinline__ void kl_apply_body(const K
   }
   if constexpr (MODE == GRAM)
     ss_finish<KW * 32>(gm, sh, a.partial, a.tickets, rhs, nblk, blk, threadIdx.x, a.scale, a.sigma,
-                       gstate<float>(a.st, rhs));
+                       a.st);
 }
 
 template <int R, int MODE> __global__ void __launch_bounds__(KW * 32) kl_apply(const __grid_constant__ KlA<R> L) {
@@ -357,7 +422,7 @@ bool carried(int step) { return step % SS_REFRESH != 0; }
 
 }  // namespace
 
-long long sl_blocks(const Grid& g) { return (long long)cdiv(g.nx + 1, BX * 2) * cdiv(g.ny + 1, BY); }
+long long sl_blocks(const Grid& g) { return (long long)cdiv(g.nx + 1, BX) * cdiv(g.ny + 1, BY); }
 
 void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2* x, const float2* b, int nu,
                      bool want_r, int B, const int* active, const GmresBufs& gb, cudaStream_t s) {
@@ -404,15 +469,15 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
     else run(std::integral_constant<int, 3>{});
     return;
   }
-  // Node-parallel: right-hand sides per block.  Stored stencils take up to
-  // four (the coefficients are then read once for them) as long as the launch
-  // keeps two blocks per SM; the other operators have nothing to share.
-  const long long nb = sl_blocks(g);
-  const bool stored = opv.kind == 2 || opv.kind == 3;
-  const int RB = stored && B >= 4 && nb * cdiv(B, 4) >= 304 ? 4 : stored && B >= 2 && nb * cdiv(B, 2) >= 304 ? 2 : 1;
+  // Node-parallel.  Stored stencils: node pairs of up to four right-hand sides
+  // per block (a coefficient is then read once for them) as long as the launch
+  // keeps two blocks per SM, else one node of one right-hand side per thread,
+  // in blocks of 512 threads once blocks of 256 would be more than two per SM
+  // (half as many records for the last block to add).  The other operators
+  // have nothing to share.
+  const long long nb = (long long)cdiv(g.nx + 1, BX * 2) * cdiv(g.ny + 1, BY);
   with_op<float>(opv, g.nx, g.ny, [&](auto op) {
     using Op = decltype(op);
-    constexpr bool S = std::is_same_v<Op, OpS<float, 2>> || std::is_same_v<Op, OpS<float, 3>>;
     auto go = [&](auto rb) {
       constexpr int N = decltype(rb)::value;
       const dim3 grd(cdiv(g.nx + 1, BX * 2), cdiv(g.ny + 1, BY), cdiv(B, N)), blk(BX, BY);
@@ -423,11 +488,25 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
         sl_apply<Op, MODE, N><<<grd, blk, 0, s>>>(a, op);
       });
     };
-    if constexpr (S) {
-      if (RB == 4) return go(std::integral_constant<int, 4>{});
-      if (RB == 2) return go(std::integral_constant<int, 2>{});
+    if constexpr (std::is_same_v<Op, OpS<float, 2>> || std::is_same_v<Op, OpS<float, 3>>) {
+      constexpr int R = std::is_same_v<Op, OpS<float, 2>> ? 2 : 3;
+      auto one = [&](auto ny) {
+        constexpr int NY = decltype(ny)::value;
+        const dim3 grd(cdiv(g.nx + 1, BX), cdiv(g.ny + 1, NY), B), blk(BX, NY);
+        steps([&](auto mode, const float2* v, float2* o) {
+          constexpr int MODE = decltype(mode)::value;
+          a.v = v;
+          a.out = o;
+          sl_one<R, MODE, NY><<<grd, blk, 0, s>>>(a, op);
+        });
+      };
+      if (B >= 4 && nb * cdiv(B, 4) >= 304) go(std::integral_constant<int, 4>{});
+      else if (B >= 2 && nb * cdiv(B, 2) >= 304) go(std::integral_constant<int, 2>{});
+      else if (sl_blocks(g) * B > 304) one(std::integral_constant<int, 16>{});
+      else one(std::integral_constant<int, 8>{});
+    } else {
+      go(std::integral_constant<int, 1>{});
     }
-    go(std::integral_constant<int, 1>{});
   });
 }
 

@@ -407,7 +407,7 @@ template <bool Z, bool VK, bool A2> __device__ __forceinline__ void ss_gram_body
   });
   __syncthreads();   // the staging rings are free: the sums reuse them
   ss_finish<SWB * 32>(g, reinterpret_cast<double*>(&stg[0][0]), a.partial, a.tickets, rhs, a.nblk, blk, threadIdx.x,
-                      a.scale, a.sigma, gstate<float>(a.st, rhs));
+                      a.scale, a.sigma, a.st);
 }
 template <bool Z, bool VK, bool A2, bool OUT>
 __device__ __forceinline__ void ss_update_body(const SmA& a, int blk, int rhs) {

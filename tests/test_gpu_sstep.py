@@ -59,3 +59,30 @@ def test_mixed_solve_matches_oracle(nx, ny, kw):
         if not kw.get("krylov"):
             assert abs(cyc[q] - ref.cycles) <= max(2, 0.1 * ref.cycles), (cyc[q], ref.cycles)
     s.close()
+
+
+@pytest.mark.parametrize("B", [5, 13, 25])
+def test_stored_stencils_share_blocks_between_right_hand_sides(B):
+    """Variable k on 257^2: the first coarse level (129^2 stored stencils) runs
+    one right-hand side per block in blocks of 512 threads (B = 5), two (13) and
+    four (25), the last group of each a partial one; a zero right-hand side
+    leaves its group's shared reduction to the others."""
+    n, h = 256, 1.0 / 256
+    k = synth.k_field(synth.chi_smooth(n, n, 2), 0.24 / h, 0.4 / h)
+    kmax = float(k.max())
+    b = synth.random_complex((B, n + 1, n + 1), 11) / h**2
+    b[2] = 0.0
+    H = ohier.build_hierarchy(n, n, h, k, 1 / kmax)
+    s = hm.Solver(n, n, h, _dev(k, torch.float64), 1 / kmax, smoother="gmres3", nu_pre=2, nu_post=2, precision="mixed",
+                  batch=B)
+    x, st, cyc, rr = s.solve(_dev(b), tol=1e-10)
+    assert st == hm.MG_OK
+    assert cyc[2] == 0 and torch.count_nonzero(x[2]).item() == 0
+    ref = ocycle.mg_solve(H, b[B - 1].ravel(), 1e-10, ocycle.CycleOptions(1, "gmres3", 2, 2, 4.5))
+    assert pu.rel2(x[B - 1].cpu().numpy(), ref.x) <= 1e-6
+    assert abs(cyc[B - 1] - ref.cycles) <= max(2, 0.1 * ref.cycles)
+    # the others by their residual with the oracle's matrix
+    for q in range(B):
+        if q != 2:
+            assert pu.rel2(H.A[0] @ x[q].cpu().numpy().ravel(), b[q].ravel()) <= 1.1e-10
+    s.close()
