@@ -1129,7 +1129,8 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
     nblk_max = std::max({nblk_max, node_blocks(c->lev[l].g), mixed && gm ? sl_blocks(c->lev[l].g) : 0LL});
     if (c->lev[l].kind == 1)
       nblk_max = std::max({nblk_max, gmres_march_blocks(c->lev[l].g, c->B),
-                           mixed && gm ? ss_march_blocks(c->lev[l].g, c->B) : 0LL});
+                           mixed && gm ? ss_march_blocks(c->lev[l].g, c->B) : 0LL,
+                           mixed ? resid_blocks(c->lev[l].g, c->B) : 0LL});
     if (c->lev[l].kind >= 4) nblk_max = std::max(nblk_max, kron_march_blocks(c->lev[l].g, c->B));
   }
   CK(dalloc(c, (void**)&c->partial, sizeof(double) * (size_t)nblk_max * c->B * NVMAX));

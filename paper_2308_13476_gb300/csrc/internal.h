@@ -113,7 +113,9 @@ __device__ __forceinline__ void stop_update(const Ctl& c, int rhs, double sumsq,
 template <class T> void launch_resnorm_stop(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                             int B, const Ctl& c, int count, cudaStream_t s);
 // Mixed path, FP64 outer loop: r = b - A x in FP64, written as float into r32
-// (same Grid), stopping test fused; and x += e (FP64 += float), masked.
+// (same Grid), stopping test fused (resid_march.cu; resid_blocks() records per
+// RHS in the partial buffer); and x += e (FP64 += float), masked.
+long long resid_blocks(const Grid& g, int B);
 void launch_resid_cast_stop(const Grid& g, const OpView<double>& op, const double2* x, const double2* b,
                             float2* r32, int B, const Ctl& c, int count, cudaStream_t s);
 void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, cudaStream_t s);

@@ -41,17 +41,6 @@ struct RsA {
 };
 
 
-struct RcA {
-  Grid g;
-  Op0<double> op;
-  const double2* x;
-  const double2* b;
-  float2* r32;
-  Ctl c;
-  int count;
-};
-
-
 struct UmA {
   Grid g;
   double2* x;
@@ -176,71 +165,6 @@ __global__ void __launch_bounds__(BX * BY) k_resnorm_stop_rag(const __grid_const
   dim3 vg;
   const RsA<T, Op>& a = L.a[rag_problem(L, blockIdx.x, vb, vg)];
   k_resnorm_stop_body<T, Op>(vb, vg, a.g, a.op, a.x, a.b, a.c, a.count);
-}
-
-// FP64 residual of the refinement loop, written in float for the next
-// complex64 correction cycle, with the stopping test fused.  This pass runs
-// at the FP64 rate, so its FP64 work is kept small: on interior nodes
-// b - A x is two FMAs per component after the neighbour sum,
-// b - d x_P + (1/h^2)(x_E + x_W + x_N + x_S), d = 4/h^2 - k^2 (boundary nodes
-// take Op0::apply5); and the norm is summed from the float residual the
-// pass writes anyway (FP32 within a thread and a warp, FP64 across warps and
-// blocks), which resolves the stopping test's relative residual to about
-// 1e-7 of itself.  The conversions to float take the integer pipe
-// (f32_from_f64_rn, the same rounding as the hardware's).
-template <bool A2>
-__device__ __forceinline__ void k_resid_cast_stop_body(uint3 vblk, dim3 vgrid, Grid g, Op0<double, A2> op, const double2* __restrict__ x, const double2* __restrict__ b, float2* __restrict__ r32, Ctl c, int count) {
-  const uint3 blockIdx = vblk;   // the block and grid inside this problem's launch
-  const dim3 gridDim = vgrid;
-  (void)blockIdx;
-  (void)gridDim;
-  __shared__ double sh[32];
-  NODE_INDEX
-  if (!c.active[rhs]) return;
-  float af = 0.f;
-  const double ih2 = op.c.inv_h2;
-  const double dconst = fma(-op.c.k, op.c.k, 4.0 * ih2);
-  if (i <= g.nx) {
-    const double2* xs = x + off;
-    FOR_ROWS {
-      if (j > g.ny) break;
-      const int p = g.at(i, j);
-      const double2 bb = b[off + p];
-      double2 r;
-      if (i > 0 && i < g.nx && j > 0 && j < g.ny) {
-        const double2 xp = xs[p], xe = xs[p + 1], xw = xs[p - 1], xn = xs[p + g.pitch], xd = xs[p - g.pitch];
-        double d = dconst;
-        if (op.kf) {
-          const double k = op.kf[j * (g.nx + 1) + i];
-          d = fma(-k, k, 4.0 * ih2);
-        }
-        const double sr = (xe.x + xw.x) + (xn.x + xd.x), si = (xe.y + xw.y) + (xn.y + xd.y);
-        r = make_double2(fma(ih2, sr, fma(-d, xp.x, bb.x)), fma(ih2, si, fma(-d, xp.y, bb.y)));
-      } else {
-        r = sub<double>(bb, op.apply(xs, p, g.pitch, i, j));
-      }
-      const float2 rf = make_float2(f32_from_f64_rn(r.x), f32_from_f64_rn(r.y));
-      r32[off + p] = rf;
-      af = fmaf(rf.x, rf.x, fmaf(rf.y, rf.y, af));
-    }
-  }
-  const float a0[1] = {af};
-  double v[1];
-  if (reduce_last<1, float>(a0, v, sh, c.partial, c.tickets, rhs, gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x) &&
-      threadIdx.x == 0 && threadIdx.y == 0)
-    stop_update(c, rhs, v[0], count);
-}
-
-template <bool A2>
-__global__ void __launch_bounds__(BX * BY) k_resid_cast_stop(Grid g, Op0<double, A2> op, const double2* __restrict__ x, const double2* __restrict__ b, float2* __restrict__ r32, Ctl c, int count) {
-  k_resid_cast_stop_body<A2>(blockIdx, gridDim, g, op, x, b, r32, c, count);
-}
-
-__global__ void __launch_bounds__(BX * BY) k_resid_cast_stop_rag(const __grid_constant__ RagLaunch<RcA> L) {
-  uint3 vb;
-  dim3 vg;
-  const RcA& a = L.a[rag_problem(L, blockIdx.x, vb, vg)];
-  k_resid_cast_stop_body(vb, vg, a.g, a.op, a.x, a.b, a.r32, a.c, a.count);
 }
 
 __device__ __forceinline__ void k_update_mixed_body(uint3 vblk, dim3 vgrid, Grid g, double2* __restrict__ x, const float2* __restrict__ e, const int* __restrict__ active) {
@@ -488,15 +412,6 @@ void launch_resnorm_stop(const Grid& g, const OpView<T>& v, const cx<T>* x, cons
     k_resnorm_stop<T, decltype(op)><<<pack_grid(g, B, PK<T>::NP), dim3(BX, BY), 0, s>>>(g, op, x, b, c, count);
   });
 }
-void launch_resid_cast_stop(const Grid& g, const OpView<double>& v, const double2* x, const double2* b, float2* r32,
-                            int B, const Ctl& c, int count, cudaStream_t s) {
-  if (v.c0.abc2)   // constants by value
-    k_resid_cast_stop<true><<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, Op0<double, true>{v.c0, v.kf, g.nx, g.ny}, x, b,
-                                                                     r32, c, count);
-  else
-    k_resid_cast_stop<false><<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, Op0<double>{v.c0, v.kf, g.nx, g.ny}, x, b, r32,
-                                                                      c, count);
-}
 void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, cudaStream_t s) {
   k_update_mixed<<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, x, e, active);
 }
@@ -581,17 +496,6 @@ void launch_update_mixed_rag(const std::vector<RagOuter>& v, cudaStream_t s) {
   rag_launch<UmA>((int)v.size(), k_update_mixed_rag, dim3(BX, BY), 0, s, [&](int q, UmA& a, int& gx, int& gy) {
     const RagOuter& O = v[q];
     a = UmA{O.g, O.x, O.e, O.c.active};
-    const dim3 d = node_grid(O.g, 1);
-    gx = (int)d.x;
-    gy = (int)d.y;
-    return true;
-  });
-}
-
-void launch_resid_cast_stop_rag(const std::vector<RagOuter>& v, int count, cudaStream_t s) {
-  rag_launch<RcA>((int)v.size(), k_resid_cast_stop_rag, dim3(BX, BY), 0, s, [&](int q, RcA& a, int& gx, int& gy) {
-    const RagOuter& O = v[q];
-    a = RcA{O.g, O.op, O.x, O.b, O.r32, O.c, count};
     const dim3 d = node_grid(O.g, 1);
     gx = (int)d.x;
     gy = (int)d.y;
