@@ -321,9 +321,7 @@ __device__ __forceinline__ bool arnoldi(Blk<T>& B, const Slab<T>& s, cx<T>* cons
     w[q] = a;
 #pragma unroll
     for (int l = 0; l <= J; ++l) {
-      const cx<T> e = cmul<T>(u[l][q], a);
-      dt[2 * l] += e.x;
-      dt[2 * l + 1] += e.y;
+      add_cmul<T>(dt[2 * l], dt[2 * l + 1], u[l][q], a);
     }
   }
   cl_push_sum<ND, NT>(B, dt);
@@ -347,16 +345,14 @@ __device__ __forceinline__ bool arnoldi(Blk<T>& B, const Slab<T>& s, cx<T>* cons
 #pragma unroll
     for (int l = 0; l <= J; ++l) {
       uu[l] = u[l][q];
-      a = sub<T>(a, mul<T>(c[l], uu[l]));
+      a = sub_mul<T>(a, c[l], uu[l]);
     }
-    et[0] += abs2<T>(a);
+    add_abs2<T>(et[0], a);
     if constexpr (J < 2) {
       u[J + 1][q] = a;
 #pragma unroll
       for (int l = 0; l <= J; ++l) {
-        const cx<T> e = cmul<T>(a, uu[l]);
-        et[1 + 2 * l] += e.x;
-        et[2 + 2 * l] += e.y;
+        add_cmul<T>(et[1 + 2 * l], et[2 + 2 * l], a, uu[l]);
       }
     }
   }
@@ -384,7 +380,7 @@ __device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool 
     if constexpr (sizeof(T) == 8) {
       cx<T>* w = B.m + B.a->ou + 3 * B.a->nu;
       T a0[1] = {T(0)};
-      CL_NODES(s) a0[0] += abs2<T>(u[0][q]);
+      CL_NODES(s) add_abs2<T>(a0[0], u[0][q]);
       cl_push_sum<1, NT>(B, a0);
       start_apply<KT, NT>(B, s, u[0]);
       cl_sync();

@@ -43,6 +43,17 @@ template <class T> __device__ __forceinline__ cx<T> cmul(cx<T> a, cx<T> b) {
   return mk<T>(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
 template <class T> __device__ __forceinline__ T abs2(cx<T> a) { return a.x * a.x + a.y * a.y; }
+// s + |a|^2, (re, im) + conj(a) b and a - c u in multiply-adds alone: two
+// instructions per real result instead of three (the complex128 kernels are
+// bound by the FP64 pipe)
+template <class T> __device__ __forceinline__ void add_abs2(T& s, cx<T> a) { s = fma(a.x, a.x, fma(a.y, a.y, s)); }
+template <class T> __device__ __forceinline__ void add_cmul(T& re, T& im, cx<T> a, cx<T> b) {
+  re = fma(a.x, b.x, fma(a.y, b.y, re));
+  im = fma(a.x, b.y, fma(-a.y, b.x, im));
+}
+template <class T> __device__ __forceinline__ cx<T> sub_mul(cx<T> a, cx<T> c, cx<T> u) {
+  return mk<T>(fma(-c.x, u.x, fma(c.y, u.y, a.x)), fma(-c.x, u.y, fma(-c.y, u.x, a.y)));
+}
 
 // Packed complex64 arithmetic: one .f32x2 instruction of the FP32 pipe for
 // both components, each rounded as by the scalar instruction (so add2, sub2,
@@ -82,9 +93,9 @@ __device__ __forceinline__ cx<T> scl_minus(T s, cx<T> a, const cx<T> (&c)[L], co
     }
     return make_float2(p.x + q.y, p.y - q.x);
   } else {
-    cx<T> u = sub<T>(scl<T>(s, a), mul<T>(c[0], v[0]));
+    cx<T> u = scl<T>(s, a);
 #pragma unroll
-    for (int l = 1; l < L; ++l) u = sub<T>(u, mul<T>(c[l], v[l]));
+    for (int l = 0; l < L; ++l) u = sub_mul<T>(u, c[l], v[l]);
     return u;
   }
 }
@@ -225,6 +236,22 @@ template <class T, bool A2 = false> struct Op0 {
     } else {
       return add<T>(a, abc2_term(xp, xe, xw, xn, xs, i, j, bx, by));
     }
+  }
+  // f A x + b with the factor folded into the two coefficients (d f and -f /
+  // h^2, which the caller's loop keeps): five instructions per component at
+  // interior nodes
+  template <bool ADD> __device__ __forceinline__ cx<T> apply_fb(T f, cx<T> b, const cx<T>* __restrict__ x, int p,
+                                                                int pitch, int i, int j) const {
+    const cx<T> xp = x[p], xe = x[p + 1], xw = x[p - 1], xn = x[p + pitch], xs = x[p - pitch];
+    if (i > 0 && i < nx && j > 0 && j < ny) {
+      const T k = kval(i, j), d = f * fma(-k, k, T(4) * c.inv_h2), q = -f * c.inv_h2;
+      const T sr = (xe.x + xw.x) + (xn.x + xs.x), si = (xe.y + xw.y) + (xn.y + xs.y);
+      if constexpr (ADD) return mk<T>(fma(q, sr, fma(d, xp.x, b.x)), fma(q, si, fma(d, xp.y, b.y)));
+      else return mk<T>(fma(d, xp.x, q * sr), fma(d, xp.y, q * si));
+    }
+    const cx<T> a = scl<T>(f, apply5(xp, xe, xw, xn, xs, i, j));
+    if constexpr (ADD) return add<T>(b, a);
+    else return a;
   }
   // the tangential term: i sum_Q c_PQ (x_P - x_Q)
   __device__ __forceinline__ cx<T> abc2_term(cx<T> xp, cx<T> xe, cx<T> xw, cx<T> xn, cx<T> xs, int i, int j, bool bx,
@@ -429,20 +456,22 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh /* [NV][32
 }
 
 // Block-wide sum of NV values of the working precision T: the warp stage runs
-// in T (shuffles), each warp's sum is widened to double once, and thread 0
-// adds the warps in double.  Fixed shape and order (reproducible).
+// in T (lane_sum over the next power of two of values: 9 adds for six values
+// instead of a tree of 5 each, the same pairs in the same order), each warp's
+// sum is widened to double once, and thread 0 adds the warps in double.
+// Fixed shape and order (reproducible).
 template <int NV, class T>
 __device__ __forceinline__ void block_sum_t(const T (&v)[NV], double* sh /* [NV][32] */, double (&out)[NV]) {
+  constexpr int P = NV > 16 ? 32 : NV > 8 ? 16 : NV > 4 ? 8 : NV > 2 ? 4 : NV;
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
   const int lane = tid & 31, warp = tid >> 5;
   const int nwarps = (blockDim.x * blockDim.y) >> 5;
+  T a[P];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    T t = v[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) sh[k * 32 + warp] = (double)t;
-  }
+  for (int k = 0; k < P; ++k) a[k] = k < NV ? v[k] : T(0);
+  const T t = lane_sum<P, T>(a, lane);
+  const int k = lane_value<P>(lane);
+  if ((lane & (32 / P - 1)) == 0 && k < NV) sh[k * 32 + warp] = (double)t;
   __syncthreads();
   warp_sums_to_thread0<NV>(sh, nwarps, warp, lane, out);
   __syncthreads();

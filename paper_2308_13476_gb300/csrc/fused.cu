@@ -73,7 +73,7 @@ __device__ __forceinline__ void k_resid_restrict_body(uint3 vblk, dim3 vgrid, Gr
         const int i = fx0 + li, j = fy0 + lj;
         const int ic = min(max(i, 0), gf.nx), jc = min(max(j, 0), gf.ny);
         const int p = gf.at(ic, jc);
-        const cx<T> r = sub<T>(bs[p], op.apply(xs, p, gf.pitch, ic, jc));
+        const cx<T> r = op.template apply_fb<true>(T(-1), bs[p], xs, p, gf.pitch, ic, jc);
         const bool in = i == ic && j == jc;
         rt[lj][li] = in ? r : mk<T>(0, 0);   // outside the grid the fine residual is zero
       }

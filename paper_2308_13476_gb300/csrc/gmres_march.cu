@@ -75,15 +75,13 @@ template <class T, int MD> struct P0 {
     if (c.own_row(t - 1)) mstore(us, c.g, c.i, t - 1, u);
 #pragma unroll
     for (int n = 0; n < NP; ++n)
-      if (c.cnt(n, t - 1)) acc[0] += abs2<T>(u.v[n]);
+      if (c.cnt(n, t - 1)) add_abs2<T>(acc[0], u.v[n]);
     if (t - 2 >= c.j0) {
       const Row<T> au = c.apply(U[Sl<S, -3>::v], U[Sl<S, -2>::v], U[Sl<S, -1>::v], t - 2);
 #pragma unroll
       for (int n = 0; n < NP; ++n)
         if (c.cnt(n, t - 2)) {
-          const cx<T> d = cmul<T>(U[Sl<S, -2>::v].v[n], au.v[n]);
-          acc[1] += d.x;
-          acc[2] += d.y;
+          add_cmul<T>(acc[1], acc[2], U[Sl<S, -2>::v].v[n], au.v[n]);
         }
     }
   }
@@ -102,15 +100,13 @@ template <class T, int MD> struct P0Z {
     const Row<T>(&U)[4] = m.F[0];
 #pragma unroll
     for (int n = 0; n < NP; ++n)
-      if (c.cnt(n, t - 1)) acc[0] += abs2<T>(U[Sl<S, -1>::v].v[n]);
+      if (c.cnt(n, t - 1)) add_abs2<T>(acc[0], U[Sl<S, -1>::v].v[n]);
     if (t - 2 >= c.j0) {
       const Row<T> au = c.apply(U[Sl<S, -3>::v], U[Sl<S, -2>::v], U[Sl<S, -1>::v], t - 2);
 #pragma unroll
       for (int n = 0; n < NP; ++n)
         if (c.cnt(n, t - 2)) {
-          const cx<T> d = cmul<T>(U[Sl<S, -2>::v].v[n], au.v[n]);
-          acc[1] += d.x;
-          acc[2] += d.y;
+          add_cmul<T>(acc[1], acc[2], U[Sl<S, -2>::v].v[n], au.v[n]);
         }
     }
   }
@@ -143,21 +139,16 @@ template <class T, int MD> struct P1 {
 #pragma unroll
     for (int n = 0; n < NP; ++n)
       if (c.cnt(n, t - 1)) {
-        acc[0] += abs2<T>(u.v[n]);
-        const cx<T> d = cmul<T>(u.v[n], V[Sl<S, -1>::v].v[n]);
-        acc[1] += d.x;
-        acc[2] += d.y;
+        add_abs2<T>(acc[0], u.v[n]);
+        add_cmul<T>(acc[1], acc[2], u.v[n], V[Sl<S, -1>::v].v[n]);
       }
     if (t - 2 >= c.j0) {
       const Row<T> au = c.apply(U[Sl<S, -3>::v], U[Sl<S, -2>::v], U[Sl<S, -1>::v], t - 2);
 #pragma unroll
       for (int n = 0; n < NP; ++n)
         if (c.cnt(n, t - 2)) {
-          const cx<T> d0 = cmul<T>(V[Sl<S, -2>::v].v[n], au.v[n]), d1 = cmul<T>(U[Sl<S, -2>::v].v[n], au.v[n]);
-          acc[3] += d0.x;
-          acc[4] += d0.y;
-          acc[5] += d1.x;
-          acc[6] += d1.y;
+          add_cmul<T>(acc[3], acc[4], V[Sl<S, -2>::v].v[n], au.v[n]);
+          add_cmul<T>(acc[5], acc[6], U[Sl<S, -2>::v].v[n], au.v[n]);
         }
     }
   }
@@ -192,26 +183,18 @@ template <class T, int MD> struct P2 {
 #pragma unroll
     for (int n = 0; n < NP; ++n)
       if (c.cnt(n, t - 1)) {
-        acc[0] += abs2<T>(u.v[n]);
-        const cx<T> d0 = cmul<T>(u.v[n], Z[Sl<S, -1>::v].v[n]), d1 = cmul<T>(u.v[n], V[Sl<S, -1>::v].v[n]);
-        acc[1] += d0.x;
-        acc[2] += d0.y;
-        acc[3] += d1.x;
-        acc[4] += d1.y;
+        add_abs2<T>(acc[0], u.v[n]);
+        add_cmul<T>(acc[1], acc[2], u.v[n], Z[Sl<S, -1>::v].v[n]);
+        add_cmul<T>(acc[3], acc[4], u.v[n], V[Sl<S, -1>::v].v[n]);
       }
     if (t - 2 >= c.j0) {
       const Row<T> au = c.apply(U[Sl<S, -3>::v], U[Sl<S, -2>::v], U[Sl<S, -1>::v], t - 2);
 #pragma unroll
       for (int n = 0; n < NP; ++n)
         if (c.cnt(n, t - 2)) {
-          const cx<T> d0 = cmul<T>(Z[Sl<S, -2>::v].v[n], au.v[n]), d1 = cmul<T>(V[Sl<S, -2>::v].v[n], au.v[n]),
-                      d2 = cmul<T>(U[Sl<S, -2>::v].v[n], au.v[n]);
-          acc[5] += d0.x;
-          acc[6] += d0.y;
-          acc[7] += d1.x;
-          acc[8] += d1.y;
-          acc[9] += d2.x;
-          acc[10] += d2.y;
+          add_cmul<T>(acc[5], acc[6], Z[Sl<S, -2>::v].v[n], au.v[n]);
+          add_cmul<T>(acc[7], acc[8], V[Sl<S, -2>::v].v[n], au.v[n]);
+          add_cmul<T>(acc[9], acc[10], U[Sl<S, -2>::v].v[n], au.v[n]);
         }
     }
   }
@@ -235,7 +218,7 @@ template <class T, int MD> struct P3 {
       if (c.cnt(n, t - 1)) {
         const cx<T> v[3] = {m.F[1][Sl<S, -1>::v].v[n], m.F[2][Sl<S, -1>::v].v[n], V[Sl<S, -1>::v].v[n]};
         const cx<T> u = scl_minus<T, 3>(s2, av.v[n], cl, v);
-        acc[0] += abs2<T>(u);
+        add_abs2<T>(acc[0], u);
       }
   }
 };

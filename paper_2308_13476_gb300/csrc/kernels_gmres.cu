@@ -74,13 +74,10 @@ __global__ void __launch_bounds__(BX * BY) g_init(Grid g, Op op, const cx<T>* __
     GROWS {
       if (j > g.ny) break;
       const int p = g.at(i0, j);
-      const Pack<T> ax = apply_pack<T>(op, x + off, p, g.pitch, i0, j);
-      Pack<T> r = load_pack(b + off, p);
+      const Pack<T> r = residual_pack<T>(op, b + off, x + off, p, g.pitch, i0, j);
 #pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        r.v[n] = sub<T>(r.v[n], ax.v[n]);
-        if (n < nv) a0[0] += abs2<T>(r.v[n]);
-      }
+      for (int n = 0; n < NP; ++n)
+        if (n < nv) add_abs2<T>(a0[0], r.v[n]);
       store_pack(u0 + off, p, r, nv);
     }
   }
@@ -104,7 +101,7 @@ __global__ void __launch_bounds__(BX * BY) g_init_zero(Grid g, const cx<T>* __re
       const Pack<T> r = load_pack(b + off, g.at(i0, j));
 #pragma unroll
       for (int n = 0; n < NP; ++n)
-        if (n < nv) a0[0] += abs2<T>(r.v[n]);
+        if (n < nv) add_abs2<T>(a0[0], r.v[n]);
     }
   }
   double v[1];
@@ -132,20 +129,14 @@ __global__ void __launch_bounds__(BX * BY) g_arn_a(Grid g, Op op, const cx<T>* _
     GROWS {
       if (j > g.ny) break;
       const int p = g.at(i0, j);
-      Pack<T> a = apply_pack<T>(op, uJ + off, p, g.pitch, i0, j);
-#pragma unroll
-      for (int n = 0; n < NP; ++n) a.v[n] = scl<T>(sJ, a.v[n]);
+      const Pack<T> a = scaled_pack<T>(op, sJ, uJ + off, p, g.pitch, i0, j);
       store_pack(w + off, p, a, nv);
 #pragma unroll
       for (int l = 0; l <= J; ++l) {
         const Pack<T> ul = load_pack(us[l] + off, p);
 #pragma unroll
         for (int n = 0; n < NP; ++n) {
-          if (n < nv) {
-            const cx<T> d = cmul<T>(ul.v[n], a.v[n]);
-            acc[2 * l] += d.x;
-            acc[2 * l + 1] += d.y;
-          }
+          if (n < nv) add_cmul<T>(acc[2 * l], acc[2 * l + 1], ul.v[n], a.v[n]);
         }
       }
     }
@@ -197,20 +188,17 @@ __device__ __forceinline__ void g_arn_b_body(uint3 vblk, dim3 vgrid, Grid g, con
       for (int l = 0; l <= J; ++l) {
         uu[l] = load_pack(us[l] + off, p);
 #pragma unroll
-        for (int n = 0; n < NP; ++n) a.v[n] = sub<T>(a.v[n], mul<T>(c[l], uu[l].v[n]));
+        for (int n = 0; n < NP; ++n) a.v[n] = sub_mul<T>(a.v[n], c[l], uu[l].v[n]);
       }
       if (un) store_pack(un + off, p, a, nv);
 #pragma unroll
       for (int n = 0; n < NP; ++n) {
         if (n >= nv) continue;
-        acc[0] += abs2<T>(a.v[n]);
+        add_abs2<T>(acc[0], a.v[n]);
         if (J < 2) {
 #pragma unroll
-          for (int l = 0; l <= J && 1 + 2 * l + 1 < NV; ++l) {
-            const cx<T> d = cmul<T>(a.v[n], uu[l].v[n]);
-            acc[1 + 2 * l] += d.x;
-            acc[2 + 2 * l] += d.y;
-          }
+          for (int l = 0; l <= J && 1 + 2 * l + 1 < NV; ++l)
+            add_cmul<T>(acc[1 + 2 * l], acc[2 + 2 * l], a.v[n], uu[l].v[n]);
         }
       }
     }

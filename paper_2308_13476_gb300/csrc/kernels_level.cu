@@ -141,11 +141,10 @@ __device__ __forceinline__ void k_resnorm_stop_body(uint3 vblk, dim3 vgrid, Grid
     FOR_ROWS {
       if (j > g.ny) break;
       const int p = g.at(i0, j);
-      const Pack<T> ax = apply_pack<T>(op, x + off, p, g.pitch, i0, j);
-      const Pack<T> bb = load_pack(b + off, p);
+      const Pack<T> r = residual_pack<T>(op, b + off, x + off, p, g.pitch, i0, j);
 #pragma unroll
       for (int n = 0; n < NP; ++n)
-        if (n < nv) a0[0] += abs2<T>(sub<T>(bb.v[n], ax.v[n]));
+        if (n < nv) add_abs2<T>(a0[0], r.v[n]);
     }
   }
   double v[1];

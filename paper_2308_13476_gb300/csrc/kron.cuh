@@ -262,7 +262,7 @@ template <class T, int R> struct KRing {
   const int last = j1 + R - 1;                                                \
   ring.prime(last);
 
-constexpr int KCH[] = {64, 48, 32, 24, 16, 12, 8};   // candidate rows per chunk
+constexpr int KCH_MIN = 8, KCH_MAX = 64;   // rows per chunk
 
 // Rows per chunk for a level: each warp marches ch + 2R rows, and the
 // launch runs in ceil(blocks / cap) rounds of the cap blocks the GPU holds
@@ -272,13 +272,13 @@ constexpr int KCH[] = {64, 48, 32, 24, 16, 12, 8};   // candidate rows per chunk
 KGeo kron_geo(const Grid& g, int B, int R, long long cap, int forced = 0) {
   KGeo k;
   k.ncw = cdiv(g.nx + 1, 32);
-  if (forced > 0) {   // a fixed height (the autotuner's axis), at least the shortest candidate
-    k.ch = std::max(forced, KCH[sizeof(KCH) / sizeof(KCH[0]) - 1]);
+  if (forced > 0) {   // a fixed height (the autotuner's axis), at least the shortest
+    k.ch = std::max(forced, KCH_MIN);
     k.nchunks = cdiv(g.ny + 1, k.ch);
     return k;
   }
   long long best = -1;
-  for (int ch : KCH) {
+  for (int ch = KCH_MAX; ch >= KCH_MIN; --ch) {
     const long long blocks = (long long)cdiv((long long)k.ncw * cdiv(g.ny + 1, ch), KW) * B;
     const long long cost = (long long)cdiv(blocks, cap) * (ch + 2 * R);
     if (best < 0 || cost < best) {

@@ -76,7 +76,7 @@ __device__ __forceinline__ void km_init_body(uint3 vblk, dim3 vgrid, Grid g, KGe
         const int p = g.at(i, m);
         const cx<T> res = sub<T>(ring.own_at(m), ring.template combine<P>(op, m));
         u0[off + p] = res;
-        a0[0] += abs2<T>(res);
+        add_abs2<T>(a0[0], res);
       }
     });
     asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(KW * 32) km_init_zero(Grid g, KGeo kg, const c
   if (has && i <= g.nx) {
     const cx<T>* bs = b + off;
 #pragma unroll 4
-    for (int m = j0; m < j1; ++m) a0[0] += abs2<T>(bs[g.at(i, m)]);
+    for (int m = j0; m < j1; ++m) add_abs2<T>(a0[0], bs[g.at(i, m)]);
   }
   double v[1];
   if (reduce_last<1, T>(a0, v, sh, partial, tickets, rhs, gridDim.x, blockIdx.x) && threadIdx.x == 0)
@@ -155,11 +155,8 @@ __device__ __forceinline__ void km_arn_a_body(uint3 vblk, dim3 vgrid, Grid g, KG
         const cx<T> a = scl<T>(sJ, ring.template combine<P>(op, m));
         w[off + p] = a;
 #pragma unroll
-        for (int l = 0; l <= J; ++l) {   // u_J is the staged vector
-          const cx<T> d = cmul<T>(l == J ? ring.staged_at(m) : us[l][p], a);
-          acc[2 * l] += d.x;
-          acc[2 * l + 1] += d.y;
-        }
+        for (int l = 0; l <= J; ++l)   // u_J is the staged vector
+          add_cmul<T>(acc[2 * l], acc[2 * l + 1], l == J ? ring.staged_at(m) : us[l][p], a);
       }
     });
     asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -182,14 +179,17 @@ __global__ void __launch_bounds__(KW * 32) km_arn_a_rag(const __grid_constant__ 
   km_arn_a_body<T, R, J>(vb, vg, a.g, a.kg, a.op, a.u0, a.u1, a.u2, a.w, a.st, a.partial, a.tickets, a.active);
 }
 
-// Blocks of the level's heaviest march (km_arn_a<T, R, 2>) resident on the
-// device at once.
+// Blocks that share the device's time in the choice of the chunk height
+// (kron_geo).  complex64: the blocks of the level's heaviest march (km_arn_a<T,
+// R, 2>) resident at once.  complex128: one per SM, because one warp per
+// scheduler already fills the FP64 pipe, so a second block on an SM doubles
+// its time (8 x 129^2, radius 3: 86 -> 56 us with one block of 9 rows per SM).
 template <class T, int R> long long kron_capacity() {
   static const long long cap = [] {
     int dev = 0, sms = 1, per = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, km_arn_a<T, R, 2>, KW * 32, 0);
+    if (sizeof(T) == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, km_arn_a<T, R, 2>, KW * 32, 0);
     cudaGetLastError();
     return (long long)std::max(per, 1) * std::max(sms, 1);
   }();
@@ -205,7 +205,7 @@ template <class T, int J> void launch_arn_b(const Grid& g, const GmresBufs& gb, 
 
 long long kron_march_blocks(const Grid& g, int B) {   // the most for any chunk height: the shortest
   (void)B;
-  return cdiv((long long)cdiv(g.nx + 1, 32) * cdiv(g.ny + 1, KCH[sizeof(KCH) / sizeof(KCH[0]) - 1]), KW);
+  return cdiv((long long)cdiv(g.nx + 1, 32) * cdiv(g.ny + 1, KCH_MIN), KW);
 }
 
 template <class T>

@@ -5,6 +5,8 @@
 // aligned.  Packs that straddle the grid's right edge store only their nodes
 // inside the grid, so the zero halo is never written.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace hmg {
@@ -66,6 +68,34 @@ template <> struct PackApply<float, Op0<float>> {
 template <class T, class Op>
 __device__ __forceinline__ Pack<T> apply_pack(const Op& op, const cx<T>* x, int p, int pitch, int i0, int j) {
   return PackApply<T, Op>::run(op, x, p, pitch, i0, j);
+}
+
+// s A x and b - A x on the pack of nodes; the complex128 fine level folds the
+// scale (the subtraction) into the stencil's coefficients.
+template <class T, class Op>
+__device__ __forceinline__ Pack<T> scaled_pack(const Op& op, T s, const cx<T>* x, int p, int pitch, int i0, int j) {
+  Pack<T> r;
+  if constexpr (sizeof(T) == 8 && (std::is_same_v<Op, Op0<T>> || std::is_same_v<Op, Op0<T, true>>)) {
+    r.v[0] = op.template apply_fb<false>(s, mk<T>(0, 0), x, p, pitch, i0, j);
+  } else {
+    r = apply_pack<T>(op, x, p, pitch, i0, j);
+#pragma unroll
+    for (int n = 0; n < PK<T>::NP; ++n) r.v[n] = scl<T>(s, r.v[n]);
+  }
+  return r;
+}
+template <class T, class Op>
+__device__ __forceinline__ Pack<T> residual_pack(const Op& op, const cx<T>* b, const cx<T>* x, int p, int pitch,
+                                                 int i0, int j) {
+  Pack<T> r = load_pack(b, p);
+  if constexpr (sizeof(T) == 8 && (std::is_same_v<Op, Op0<T>> || std::is_same_v<Op, Op0<T, true>>)) {
+    r.v[0] = op.template apply_fb<true>(T(-1), r.v[0], x, p, pitch, i0, j);
+  } else {
+    const Pack<T> ax = apply_pack<T>(op, x, p, pitch, i0, j);
+#pragma unroll
+    for (int n = 0; n < PK<T>::NP; ++n) r.v[n] = sub<T>(r.v[n], ax.v[n]);
+  }
+  return r;
 }
 
 }  // namespace hmg
