@@ -20,7 +20,7 @@
 // in registers, so that a few warps per SM keep the pipe busy.  Against the
 // node-parallel form with ten FP64 instructions per node: 64 x 1025^2 1740 ->
 // 1212 us (87 % of the pipe's measured rate), 16 x 513^2 with a k field 143 ->
-// 104 us, one 1025^2 46 -> 27 us; 64 right-hand sides on 1025^2 623 -> 576 ms.  The nodes
+// 104 us, one 1025^2 46 -> 32 us; 64 right-hand sides on 1025^2 623 -> 576 ms.  The nodes
 // of the boundary ring take Op0::apply5 in warps of their own: their rows
 // cost three times as much and would hold up every edge strip.
 #include "internal.h"
