@@ -355,8 +355,14 @@ template <class T> struct Emit {
         std::swap(cur[l], oth[l]);
       }
     } else if (c->opt.smoother == 0) {
+      // a zero iterate needs no application, and a Kronecker-form level takes
+      // its sweeps as column marches (a third of OpK::apply's arithmetic): 8 x
+      // 257^2, radius 2, 17.1 -> 4.6 and 9.8 us, 129^2, radius 3, 10.9 -> 3.6 and 10.3 us
+      const bool march = c->opt.fuse && op.kind >= 4 && use_march(c, l);
       for (int q = 0; q < nu; ++q) {
-        launch_jacobi<T>(g, op, cur[l], V.b, oth[l], c->B, c->active, s);
+        if (z && q == 0) launch_jacobi<T>(g, op, nullptr, V.b, oth[l], c->B, c->active, s);
+        else if (march) launch_kron_jacobi<T>(g, op, cur[l], V.b, oth[l], c->B, c->active, c->opt.kron_chunk, s);
+        else launch_jacobi<T>(g, op, cur[l], V.b, oth[l], c->B, c->active, s);
         std::swap(cur[l], oth[l]);
       }
     } else {
@@ -406,7 +412,10 @@ template <class T> struct Emit {
     } else if (l + 1 >= lc && c->coop_grid == 0) {
       cycle(l + 1);   // the cluster launch starts from x = 0 and makes all visits
     } else {
-      cudaMemsetAsync(cur[l + 1], 0, sizeof(cx<T>) * (size_t)gc.vstride * c->B, s);
+      // the level's first smoothing takes a zero iterate without reading it
+      // (complex128 GMRES(3) reads it in its update)
+      const bool unread = c->opt.nu_pre > 0 && l + 1 < lc && (c->opt.smoother == 0 || c->opt.precision > 0);
+      if (!unread) cudaMemsetAsync(cur[l + 1], 0, sizeof(cx<T>) * (size_t)gc.vstride * c->B, s);
       zx[l + 1] = 1;
       for (int q = 0; q < c->opt.cycle; ++q) cycle(l + 1);
     }
@@ -741,6 +750,7 @@ template <class T> static mg_status profile_t(mg_ctx* h, int what, int level, in
     double gop = 0;   // operator bytes per node and RHS read by one pass
     if (level == 0) gop = op.kf ? sizeof(T) / (double)h->B : 0.0;
     else if (h->lev[level].kind <= 3) gop = opbytes - e / h->B;   // stencil without the inverse diagonal
+    // counted for the Arnoldi form (the complex64 levels' s-step form moves less):
     // fine-level row marches + update 16, complex64 13 (no M3: u3's norm from the Gram form); Kronecker column
     // marches, complex64 (two fused passes, no closing g_arn_b<2>) 19; else 28, complex64 23 (no g_arn_b<2>,
     // and g_arn_a<2> stores no w)

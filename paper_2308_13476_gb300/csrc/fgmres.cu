@@ -201,6 +201,47 @@ __global__ void __launch_bounds__(FTHREADS) k_fg_restart(FgArgs a, cx<T>* __rest
 
 // ------------------------------------------------------------------ dots (MGS coefficients)
 
+// Gram row jj and the MGS coefficients of column jj (v_i = s_i u_i) from the
+// sums of the dots pass: h_q = <v_q, w> - sum_{l<q} h_l <v_q, v_l>.  One warp of
+// the last block, lane q on h_q (jj < 32): h_l is final after l rounds and is
+// passed on by a shuffle.  The launch waits for this chain: with one thread on
+// the jj^2 / 2 products in global memory the pass took 98 us on average over a
+// restart of 20 (8 x 513^2), now 84 us.
+__device__ void fg_mgs(const FgArgs& a, int rhs, int jj, const double* tot, int lane) {
+  const FgLayout L{a.m};
+  double* S = a.S + (long long)rhs * a.sd;
+  const double sjj = S[L.s(jj)], sq = lane <= jj ? S[L.s(lane)] : 0.0;
+  const double* own = tot + 2 * (jj + 1);   // <u_l, u_jj>
+  if (lane < jj) {   // <v_jj, v_l> = s_jj s_l conj(<u_l, u_jj>)
+    const double f = sjj * sq;
+    S[L.gram(jj, lane)] = f * own[2 * lane];
+    S[L.gram(jj, lane) + 1] = -f * own[2 * lane + 1];
+  }
+  __syncwarp();
+  double hr = lane <= jj ? sq * tot[2 * lane] : 0.0, hi = lane <= jj ? sq * tot[2 * lane + 1] : 0.0;
+  constexpr int G = 8;   // Gram entries loaded ahead
+  for (int l0 = 0; l0 < jj; l0 += G) {
+    double2 gm[G];
+#pragma unroll
+    for (int e = 0; e < G; ++e)
+      gm[e] = l0 + e < lane && lane <= jj ? *reinterpret_cast<const double2*>(S + L.gram(lane, l0 + e))
+                                          : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int e = 0; e < G; ++e) {
+      const int l = min(l0 + e, 31);
+      const double ar = __shfl_sync(0xffffffffu, hr, l), ai = __shfl_sync(0xffffffffu, hi, l);
+      if (l0 + e < lane && lane <= jj) {
+        hr -= ar * gm[e].x - ai * gm[e].y;
+        hi -= ar * gm[e].y + ai * gm[e].x;
+      }
+    }
+  }
+  if (lane <= jj) {
+    S[L.h(jj, lane)] = hr;
+    S[L.h(jj, lane) + 1] = hi;
+  }
+}
+
 template <class T, bool A2>
 __global__ void __launch_bounds__(FTHREADS, FG_MINB<T>) k_fg_dots(FgArgs a, const cx<T>* __restrict__ z, int jj) {
   __shared__ double red[FNV][FBY];
@@ -274,28 +315,7 @@ __global__ void __launch_bounds__(FTHREADS, FG_MINB<T>) k_fg_dots(FgArgs a, cons
   }
   __syncthreads();
   if (!fg_reduce(a, rhs, nval, mine, tot)) return;
-  if (tid) return;
-  // Gram row jj, then the MGS coefficients of column jj (v_i = s_i u_i)
-  const FgLayout L{a.m};
-  double* S = a.S + (long long)rhs * a.sd;
-  const double sjj = S[L.s(jj)];
-  for (int l = 0; l < jj; ++l) {   // <v_jj, v_l> = s_jj s_l conj(<u_l, u_jj>)
-    const double f = sjj * S[L.s(l)];
-    S[L.gram(jj, l)] = f * tot[2 * (jj + 1) + 2 * l];
-    S[L.gram(jj, l) + 1] = -f * tot[2 * (jj + 1) + 2 * l + 1];
-  }
-  for (int q = 0; q <= jj; ++q) {
-    const double sq = S[L.s(q)];
-    double hr = sq * tot[2 * q], hi = sq * tot[2 * q + 1];
-    for (int l = 0; l < q; ++l) {
-      const double ar = S[L.h(jj, l)], ai = S[L.h(jj, l) + 1];
-      const double gr = S[L.gram(q, l)], gi = S[L.gram(q, l) + 1];
-      hr -= ar * gr - ai * gi;
-      hi -= ar * gi + ai * gr;
-    }
-    S[L.h(jj, q)] = hr;
-    S[L.h(jj, q) + 1] = hi;
-  }
+  if (tid < 32) fg_mgs(a, rhs, jj, tot, tid);
 }
 
 // ------------------------------------------------------------------ orth (new basis vector, Givens)
@@ -318,64 +338,80 @@ __device__ void givens(double2 a, double2 b, double& c, double2& s) {
   }
 }
 
-__device__ void fg_finish_step(const FgArgs& a, int rhs, int jj, double sumsq) {
+__device__ __forceinline__ double2 shfl2(double2 v, int l) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+
+// End of Arnoldi step jj, by one warp of the last block: the rotations, the
+// residual estimate and, when the restart cycle ends, the back substitution.
+// Lane i holds entry i of the new column and of the earlier rotations (loaded
+// at once); every lane walks the chain of rotations on shuffled values.
+__device__ void fg_finish_step(const FgArgs& a, int rhs, int jj, double sumsq, int lane) {
   const FgLayout L{a.m};
   double* S = a.S + (long long)rhs * a.sd;
-  const double nrm = sqrt(sumsq);
-  const double beta = S[L.beta()];
+  auto at = [&](int o) { return *reinterpret_cast<const double2*>(S + o); };
+  const double2 z = make_double2(0.0, 0.0);
+  const double2 hv = lane <= jj ? at(L.h(jj, lane)) : z;
+  const double cl = lane < jj ? S[L.cs(lane)] : 0.0;
+  const double2 sl = lane < jj ? make_double2(S[L.sn(lane)], S[L.sn(lane) + 1]) : z;
+  const double2 gj = make_double2(S[L.g(jj)], S[L.g(jj) + 1]);
+  const double beta = S[L.beta()], nrm = sqrt(sumsq);
+  const int kmax = a.kst[2 * rhs + 1];
   const bool brk = nrm <= 1e-14 * beta;
-  double2 hc[FG_MAXM + 1];
-  for (int i = 0; i <= jj; ++i) hc[i] = make_double2(S[L.h(jj, i)], S[L.h(jj, i) + 1]);
-  hc[jj + 1] = make_double2(nrm, 0.0);
+  double2 x0 = shfl2(hv, 0), mine = z;
   for (int i = 0; i < jj; ++i) {   // the earlier rotations on the new column
-    const double c = S[L.cs(i)];
-    const double2 sn = make_double2(S[L.sn(i)], S[L.sn(i) + 1]);
-    const double2 x0 = hc[i], x1 = hc[i + 1];
-    hc[i] = add<double>(scl<double>(c, x0), mul<double>(sn, x1));
-    hc[i + 1] = sub<double>(scl<double>(c, x1), cmul<double>(sn, x0));   // -conj(s) a + c b
+    const double c = __shfl_sync(0xffffffffu, cl, i);
+    const double2 sn = shfl2(sl, i), x1 = shfl2(hv, i + 1);
+    if (lane == i) mine = add<double>(scl<double>(c, x0), mul<double>(sn, x1));
+    x0 = sub<double>(scl<double>(c, x1), cmul<double>(sn, x0));   // -conj(s) a + c b
   }
   double c;
   double2 sn;
-  givens(hc[jj], hc[jj + 1], c, sn);
-  hc[jj] = add<double>(scl<double>(c, hc[jj]), mul<double>(sn, hc[jj + 1]));
-  hc[jj + 1] = make_double2(0.0, 0.0);
-  S[L.cs(jj)] = c;
-  S[L.sn(jj)] = sn.x;
-  S[L.sn(jj) + 1] = sn.y;
-  for (int i = 0; i <= jj; ++i) {
-    S[L.h(jj, i)] = hc[i].x;
-    S[L.h(jj, i) + 1] = hc[i].y;
+  const double2 x1 = make_double2(nrm, 0.0);
+  givens(x0, x1, c, sn);
+  if (lane == jj) mine = add<double>(scl<double>(c, x0), mul<double>(sn, x1));
+  if (lane <= jj) {
+    S[L.h(jj, lane)] = mine.x;
+    S[L.h(jj, lane) + 1] = mine.y;
   }
-  const double2 gj = make_double2(S[L.g(jj)], S[L.g(jj) + 1]);
   const double2 g1 = cmul<double>(sn, gj);   // conj(s) g_j
-  S[L.g(jj + 1)] = -g1.x;
-  S[L.g(jj + 1) + 1] = -g1.y;
-  S[L.g(jj)] = c * gj.x;
-  S[L.g(jj) + 1] = c * gj.y;
   const double est = hypot(g1.x, g1.y) / a.bnorm[rhs];
   const int k = jj + 1;
-  a.kst[2 * rhs] = k;
-  const int cy = ++a.cycles[rhs];
-  if (cy <= a.hist_len) a.hist[(long long)rhs * a.hist_len + cy - 1] = est;
-  if (brk || est <= a.tol || k >= a.kst[2 * rhs + 1]) {
-    // y = R^{-1} g by back substitution over the k rotated columns
-    for (int i = k - 1; i >= 0; --i) {
-      double2 t = make_double2(S[L.g(i)], S[L.g(i) + 1]);
-      for (int l = i + 1; l < k; ++l) {
-        const double2 r = make_double2(S[L.h(l, i)], S[L.h(l, i) + 1]);
-        const double2 yl = make_double2(S[L.y(l)], S[L.y(l) + 1]);
-        t = sub<double>(t, mul<double>(r, yl));
-      }
-      const double2 d = make_double2(S[L.h(i, i)], S[L.h(i, i) + 1]);
-      const double dd = d.x * d.x + d.y * d.y;
-      const double2 yi = make_double2((t.x * d.x + t.y * d.y) / dd, (t.y * d.x - t.x * d.y) / dd);
-      S[L.y(i)] = yi.x;
-      S[L.y(i) + 1] = yi.y;
+  const bool end = brk || est <= a.tol || k >= kmax;
+  if (lane == 0) {
+    S[L.cs(jj)] = c;
+    S[L.sn(jj)] = sn.x;
+    S[L.sn(jj) + 1] = sn.y;
+    S[L.g(jj + 1)] = -g1.x;
+    S[L.g(jj + 1) + 1] = -g1.y;
+    S[L.g(jj)] = c * gj.x;
+    S[L.g(jj) + 1] = c * gj.y;
+    a.kst[2 * rhs] = k;
+    const int cy = ++a.cycles[rhs];
+    if (cy <= a.hist_len) a.hist[(long long)rhs * a.hist_len + cy - 1] = est;
+    if (end) {
+      a.active[rhs] = 0;
+      atomicSub(a.n_active, 1);
+    } else {
+      S[L.s(k)] = 1.0 / nrm;
     }
-    a.active[rhs] = 0;
-    atomicSub(a.n_active, 1);
-  } else {
-    S[L.s(k)] = 1.0 / nrm;
+  }
+  if (!end) return;
+  __syncwarp();
+  // y = R^{-1} g by back substitution over the k rotated columns, lane i on y_i
+  double2 t = lane < k ? make_double2(S[L.g(lane)], S[L.g(lane) + 1]) : z, y = z;
+  const double2 d = lane < k ? at(L.h(lane, lane)) : make_double2(1.0, 0.0);
+  const double dd = d.x * d.x + d.y * d.y;
+#pragma unroll 4
+  for (int l = k - 1; l >= 0; --l) {
+    const double2 r = lane < l ? at(L.h(l, lane)) : z;
+    if (lane == l) y = make_double2((t.x * d.x + t.y * d.y) / dd, (t.y * d.x - t.x * d.y) / dd);
+    const double2 yl = shfl2(y, l);
+    if (lane < l) t = sub<double>(t, mul<double>(r, yl));
+  }
+  if (lane < k) {
+    S[L.y(lane)] = y.x;
+    S[L.y(lane) + 1] = y.y;
   }
 }
 
@@ -452,7 +488,7 @@ __global__ void __launch_bounds__(FTHREADS, FG_MINB<T>) k_fg_orth(FgArgs a, int 
   }
   __syncthreads();
   if (!fg_reduce(a, rhs, 1, mine, tot)) return;
-  if (tid == 0) fg_finish_step(a, rhs, jj, tot[0]);
+  if (tid < 32) fg_finish_step(a, rhs, jj, tot[0], tid);
 }
 
 // ------------------------------------------------------------------ update

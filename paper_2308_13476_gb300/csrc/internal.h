@@ -69,6 +69,7 @@ template <class T> void launch_residual(const Grid& g, const OpView<T>& op, cons
                                         cx<T>* r, int B, const int* active, cudaStream_t s);
 template <class T> void launch_apply(const Grid& g, const OpView<T>& op, const cx<T>* x, cx<T>* y, int B,
                                      const int* active, cudaStream_t s);
+// x = null: x is zero (the sweep is xout = (omega diag A)^{-1} b).
 template <class T> void launch_jacobi(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                       cx<T>* xout, int B, const int* active, cudaStream_t s);
 // Per-solve control block of the stopping test (device arrays, one entry per
@@ -221,6 +222,9 @@ template <class T> void gmres_smooth_kron(const Grid& g, const OpView<T>& op, cx
 // the restriction then reads; kron_ch as in GmresBufs).
 template <class T> void launch_kron_residual(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                              cx<T>* r, int B, const int* active, int kron_ch, cudaStream_t s);
+// A weighted-Jacobi sweep on a Kronecker-form level as a column march.
+template <class T> void launch_kron_jacobi(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
+                                           cx<T>* xout, int B, const int* active, int kron_ch, cudaStream_t s);
 
 // Steps of the small levels' part of a cycle, walked by the cooperative
 // interpreter (coop.cu).

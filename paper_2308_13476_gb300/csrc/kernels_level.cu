@@ -105,8 +105,9 @@ __global__ void __launch_bounds__(BX * BY) k_apply(Grid g, Op op, const cx<T>* _
   }
 }
 
-// x_out = x + (omega diag A)^{-1} (b - A x)   (one weighted-Jacobi sweep)
-template <class T, class Op>
+// x_out = x + (omega diag A)^{-1} (b - A x)   (one weighted-Jacobi sweep); Z: x
+// is zero and not read, which is the same value without the application
+template <class T, class Op, bool Z>
 __global__ void __launch_bounds__(BX * BY) k_jacobi(Grid g, Op op, const cx<T>* __restrict__ x,
                                                     const cx<T>* __restrict__ b, cx<T>* __restrict__ xo,
                                                     const int* __restrict__ active) {
@@ -116,12 +117,20 @@ __global__ void __launch_bounds__(BX * BY) k_jacobi(Grid g, Op op, const cx<T>* 
   FOR_ROWS {
     if (j > g.ny) break;
     const int p = g.at(i0, j);
-    const Pack<T> ax = apply_pack<T>(op, x + off, p, g.pitch, i0, j);
     const Pack<T> bb = load_pack(b + off, p);
-    Pack<T> xv = load_pack(x + off, p);
+    Pack<T> xv, r;
+    if constexpr (Z) {
 #pragma unroll
-    for (int n = 0; n < NP; ++n)
-      xv.v[n] = fma_c<T>(op.diag_inv(min(i0 + n, g.nx), j), sub<T>(bb.v[n], ax.v[n]), xv.v[n]);
+      for (int n = 0; n < NP; ++n) xv.v[n] = mk<T>(0, 0);
+      r = bb;
+    } else {
+      xv = load_pack(x + off, p);
+      const Pack<T> ax = apply_pack<T>(op, x + off, p, g.pitch, i0, j);
+#pragma unroll
+      for (int n = 0; n < NP; ++n) r.v[n] = sub<T>(bb.v[n], ax.v[n]);
+    }
+#pragma unroll
+    for (int n = 0; n < NP; ++n) xv.v[n] = fma_c<T>(op.diag_inv(min(i0 + n, g.nx), j), r.v[n], xv.v[n]);
     store_pack(xo + off, p, xv, nv);
   }
 }
@@ -401,7 +410,9 @@ template <class T>
 void launch_jacobi(const Grid& g, const OpView<T>& v, const cx<T>* x, const cx<T>* b, cx<T>* xo, int B,
                    const int* active, cudaStream_t s) {
   with_op<T>(v, g.nx, g.ny, [&](auto op) {
-    k_jacobi<T, decltype(op)><<<pack_grid(g, B, PK<T>::NP), dim3(BX, BY), 0, s>>>(g, op, x, b, xo, active);
+    const dim3 grd = pack_grid(g, B, PK<T>::NP), blk(BX, BY);
+    if (x) k_jacobi<T, decltype(op), false><<<grd, blk, 0, s>>>(g, op, x, b, xo, active);
+    else k_jacobi<T, decltype(op), true><<<grd, blk, 0, s>>>(g, op, x, b, xo, active);
   });
 }
 template <class T>

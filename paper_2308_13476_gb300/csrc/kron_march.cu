@@ -43,10 +43,11 @@ template <class T, int R> struct KmA {
   const int* active;
 };
 
-// u0 = b - A x, partial |u0|^2 (as g_init)
-// NRM = false: only u0 = b - A x (the residual before the restriction; no
-// norm, no state)
-template <class T, int R, bool NRM = true>
+// What km_init leaves: u0 = b - A x and partial |u0|^2 (as g_init), only u0
+// (the residual before the restriction; no norm, no state), or a weighted
+// Jacobi sweep u0 = x + (omega diag A)^{-1} (b - A x)
+enum { KM_NORM = 0, KM_RES = 1, KM_JACOBI = 2 };
+template <class T, int R, int OUT = KM_NORM>
 __device__ __forceinline__ void km_init_body(uint3 vblk, dim3 vgrid, Grid g, KGeo kg, OpK<T, R> op, const cx<T>* __restrict__ x, const cx<T>* __restrict__ b, cx<T>* __restrict__ u0, double* st, double* partial, unsigned* tickets, const int* __restrict__ active) {
   const uint3 blockIdx = vblk;   // the block and grid inside this problem's launch
   const dim3 gridDim = vgrid;
@@ -74,14 +75,15 @@ __device__ __forceinline__ void km_init_body(uint3 vblk, dim3 vgrid, Grid g, KGe
       const int m = r - R;
       if (m >= j0 && col) {
         const int p = g.at(i, m);
-        const cx<T> res = sub<T>(ring.own_at(m), ring.template combine<P>(op, m));
+        cx<T> res = sub<T>(ring.own_at(m), ring.template combine<P>(op, m));
+        if constexpr (OUT == KM_JACOBI) res = fma_c<T>(op.diag_inv(i, m), res, ring.staged_at(m));
         u0[off + p] = res;
-        add_abs2<T>(a0[0], res);
+        if constexpr (OUT == KM_NORM) add_abs2<T>(a0[0], res);
       }
     });
     asm volatile("cp.async.wait_all;\n" ::: "memory");
   }
-  if constexpr (NRM) {
+  if constexpr (OUT == KM_NORM) {
     double v[1];
     if (reduce_last<1, T>(a0, v, sh, partial, tickets, rhs, nblk, blk) && threadIdx.x == 0)
       fin_init<T>(gstate<T>(st, rhs), v);
@@ -115,9 +117,9 @@ __global__ void __launch_bounds__(KW * 32) km_init_zero(Grid g, KGeo kg, const c
     fin_init<T>(gstate<T>(st, rhs), v);
 }
 
-template <class T, int R, bool NRM = true>
+template <class T, int R, int OUT = KM_NORM>
 __global__ void __launch_bounds__(KW * 32) km_init(Grid g, KGeo kg, OpK<T, R> op, const cx<T>* __restrict__ x, const cx<T>* __restrict__ b, cx<T>* __restrict__ u0, double* st, double* partial, unsigned* tickets, const int* __restrict__ active) {
-  km_init_body<T, R, NRM>(blockIdx, gridDim, g, kg, op, x, b, u0, st, partial, tickets, active);
+  km_init_body<T, R, OUT>(blockIdx, gridDim, g, kg, op, x, b, u0, st, partial, tickets, active);
 }
 
 template <class T, int R>
@@ -243,17 +245,30 @@ void gmres_smooth_kron(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<T
   else run(kron_op<T, 3>(opv, g.nx, g.ny), std::integral_constant<int, 3>{});
 }
 
-template <class T>
-void launch_kron_residual(const Grid& g, const OpView<T>& opv, const cx<T>* x, const cx<T>* b, cx<T>* r, int B,
-                          const int* active, int kron_ch, cudaStream_t s) {
+namespace {
+template <int OUT, class T>
+void kron_pass(const Grid& g, const OpView<T>& opv, const cx<T>* x, const cx<T>* b, cx<T>* r, int B, const int* active,
+               int kron_ch, cudaStream_t s) {
   auto run = [&](auto op, auto rad) {
     constexpr int R = decltype(rad)::value;
     const KGeo kg = kron_geo(g, B, R, kron_capacity<T, R>(), kron_ch);
     const dim3 grd(cdiv((long long)kg.ncw * kg.nchunks, KW), 1, B);
-    km_init<T, R, false><<<grd, KW * 32, 0, s>>>(g, kg, op, x, b, r, nullptr, nullptr, nullptr, active);
+    km_init<T, R, OUT><<<grd, KW * 32, 0, s>>>(g, kg, op, x, b, r, nullptr, nullptr, nullptr, active);
   };
   if (opv.kind == 4) run(kron_op<T, 2>(opv, g.nx, g.ny), std::integral_constant<int, 2>{});
   else run(kron_op<T, 3>(opv, g.nx, g.ny), std::integral_constant<int, 3>{});
+}
+}  // namespace
+
+template <class T>
+void launch_kron_residual(const Grid& g, const OpView<T>& opv, const cx<T>* x, const cx<T>* b, cx<T>* r, int B,
+                          const int* active, int kron_ch, cudaStream_t s) {
+  kron_pass<KM_RES, T>(g, opv, x, b, r, B, active, kron_ch, s);
+}
+template <class T>
+void launch_kron_jacobi(const Grid& g, const OpView<T>& opv, const cx<T>* x, const cx<T>* b, cx<T>* xo, int B,
+                        const int* active, int kron_ch, cudaStream_t s) {
+  kron_pass<KM_JACOBI, T>(g, opv, x, b, xo, B, active, kron_ch, s);
 }
 
 // The same smoothing steps on every problem of a ragged batch (the problems'
@@ -303,6 +318,10 @@ template void launch_kron_residual<double>(const Grid&, const OpView<double>&, c
                                            double2*, int, const int*, int, cudaStream_t);
 template void launch_kron_residual<float>(const Grid&, const OpView<float>&, const float2*, const float2*, float2*,
                                           int, const int*, int, cudaStream_t);
+template void launch_kron_jacobi<double>(const Grid&, const OpView<double>&, const double2*, const double2*, double2*,
+                                         int, const int*, int, cudaStream_t);
+template void launch_kron_jacobi<float>(const Grid&, const OpView<float>&, const float2*, const float2*, float2*, int,
+                                        const int*, int, cudaStream_t);
 template void gmres_smooth_kron<double>(const Grid&, const OpView<double>&, double2*, const double2*, int, int,
                                         const int*, const GmresBufs&, cudaStream_t);
 
