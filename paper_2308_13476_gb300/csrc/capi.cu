@@ -553,24 +553,25 @@ template <class T> static bool cluster_plan(mg_ctx* c, int lc, int C, std::vecto
   a.x_zero = lc > 0 || c->opt.precision > 0 || c->opt.krylov > 0;
   z[lc] = a.x_zero != 0;
   steps.clear();
-  auto smooth = [&](int l, int nu) {
+  const bool left = sizeof(T) == 4 && c->opt.smoother == 1 && c->opt.nu_pre > 0;   // pre-smoothing leaves the residual
+  auto smooth = [&](int l, int nu, bool keep) {
     if (nu <= 0) return;
-    steps.push_back(ClStep{c->opt.smoother == 0 ? CL_JACOBI : CL_GMRES, l - lc, nu, z[l]});
+    steps.push_back(ClStep{c->opt.smoother == 0 ? CL_JACOBI : CL_GMRES, l - lc, nu, z[l], keep});
     z[l] = 0;
   };
   auto cycle = [&](auto&& self, int l) -> void {
     if (l == L - 1) {
-      steps.push_back(ClStep{CL_COARSE, l - lc, 0, 0});
+      steps.push_back(ClStep{CL_COARSE, l - lc, 0, 0, 0});
       return;
     }
-    smooth(l, c->opt.nu_pre);
-    steps.push_back(ClStep{CL_RESTRICT, l - lc, 0, 0});
+    smooth(l, c->opt.nu_pre, left);
+    steps.push_back(ClStep{CL_RESTRICT, l - lc, 0, 0, left});
     z[l + 1] = 1;
     const int visits = l + 1 == L - 1 ? 1 : c->opt.cycle;
     for (int q = 0; q < visits; ++q) self(self, l + 1);
-    steps.push_back(ClStep{CL_PROLONG, l - lc, 0, 0});
+    steps.push_back(ClStep{CL_PROLONG, l - lc, 0, 0, 0});
     z[l] = 0;
-    smooth(l, c->opt.nu_post);
+    smooth(l, c->opt.nu_post, false);
   };
   const int visits = lc == 0 || lc == L - 1 ? 1 : c->opt.cycle;
   for (int q = 0; q < visits; ++q) cycle(cycle, lc);

@@ -29,7 +29,8 @@
 // GMRES(3): complex128 in the Arnoldi form of the grid-wide kernels
 // (gmres.cuh).  complex64 in the s-step form of sstep.cuh: the basis r, B r,
 // B^2 r, B^3 r without sums in between, one sum of its Gram matrix, and the
-// 3 x 3 normal equations: five barriers per step instead of nine.
+// 3 x 3 normal equations: four barriers per step instead of nine (five where
+// the residual is formed afresh).
 //
 // The chain is latency-bound in complex64 (a phase is a barrier of about 0.3
 // us and a few hundred clocks of work) and bound by the SMs' FP64 pipes in
@@ -39,7 +40,11 @@
 // complex64 on 81^2 8.4 -> 3.0 ms and on 1025^2 112 -> 78.9 ms (one
 // right-hand side), FP64 8 x 513^2 521 -> 392 ms, 16 ragged problems
 // 182 -> 117 ms.
+// Carrying the residual between complex64 steps (16 -> 10 applications per
+// V(2,2) cycle and level): one 1025^2 right-hand side 48.2 -> 46.0 ms, 81^2
+// 3.02 -> 2.94 ms, 16 ragged problems 71.5 -> 68.8 ms.
 #include <algorithm>
+#include <mutex>
 
 #include "gmres.cuh"
 #include "internal.h"
@@ -365,16 +370,19 @@ __device__ __forceinline__ bool arnoldi(Blk<T>& B, const Slab<T>& s, cx<T>* cons
   return true;
 }
 
-// nu GMRES(3) steps; z: x is zero on entry, so that the first step's u0 is b.
+// nu GMRES(3) steps; z: x is zero on entry, so that the first step's u0 is b;
+// left (complex64): leave b - A x in u0.  complex64 steps after the first take
+// the residual that the previous update formed by linearity (sstep.cuh): ten
+// applications per V(2,2) cycle and level instead of sixteen.
 template <class KT, int NT, class T>
-__device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool z) {
+__device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool z, bool left) {
   cx<T>* x = B.m + s.L->ox;
   const cx<T>* b = B.m + s.L->ob;
   cx<T>* const u[3] = {B.m + B.a->ou, B.m + B.a->ou + B.a->nu, B.m + B.a->ou + 2 * B.a->nu};
   for (int step = 0; step < nu; ++step) {
     if (z && step == 0) {
       CL_NODES(s) u[0][q] = b[q];
-    } else {
+    } else if (sizeof(T) == 8 || !ss_carried(step)) {
       residual<KT, NT>(B, s, u[0]);
     }
     if constexpr (sizeof(T) == 8) {
@@ -407,6 +415,8 @@ __device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool 
       __syncthreads();
     } else {
       const T sc = s.L->scale, sg = s.L->sigma;
+      cx<T>* v3s = B.m + B.a->ou + 3 * B.a->nu;
+      const bool nr = step + 1 < nu ? ss_carried(step + 1) : left;   // the next residual is wanted
       T gm[SS_NV];
 #pragma unroll
       for (int k = 0; k < SS_NV; ++k) gm[k] = T(0);
@@ -425,6 +435,7 @@ __device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool 
             const cx<T> a = combine<KT>(B, s, jl, i), v2 = u[2][q];
             const cx<T> v3 = mk<T>(fma(sc, a.x, -sg * v2.x), fma(sc, a.y, -sg * v2.y));
             ss_gram_add(gm, u[0][q], u[1][q], v2, v3);
+            if (nr) v3s[q] = v3;
           }
         }
       }
@@ -436,11 +447,20 @@ __device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool 
       cx<T> y[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) y[k] = mk<T>(B.S[2 * k], B.S[2 * k + 1]);
+      cx<T> c[4];
+      ss_residual_coef(y, T(1) / sc, sg, c);
       CL_NODES(s) {
         cx<T> e = z && step == 0 ? mk<T>(0, 0) : x[q];
+        const cx<T> v[3] = {u[0][q], u[1][q], u[2][q]};
 #pragma unroll
-        for (int k = 0; k < 3; ++k) e = fma_c<T>(y[k], u[k][q], e);
+        for (int k = 0; k < 3; ++k) e = fma_c<T>(y[k], v[k], e);
         x[q] = e;
+        if (nr) {
+          cx<T> r = mul<T>(c[0], v[0]);
+          r = fma_c<T>(c[1], v[1], r);
+          r = fma_c<T>(c[2], v[2], r);
+          u[0][q] = fma_c<T>(c[3], v3s[q], r);
+        }
       }
       __syncthreads();
     }
@@ -449,12 +469,13 @@ __device__ __forceinline__ void gmres(Blk<T>& B, const Slab<T>& s, int nu, bool 
 
 // --------------------------------------------------------------- transfers
 
-// b_{l+1} = R (b - A x) and x_{l+1} = 0
-template <class KT, int NT, class T> __device__ __forceinline__ void restrict_to(Blk<T>& B, const Slab<T>& s, int l) {
+// b_{l+1} = R (b - A x) and x_{l+1} = 0; left: b - A x is in u0
+template <class KT, int NT, class T>
+__device__ __forceinline__ void restrict_to(Blk<T>& B, const Slab<T>& s, int l, bool left) {
   const ClLev<T>& L = *s.L;
   cx<T>* r = B.m + B.a->ou;
   cx<T>* t = B.m + B.a->ou + B.a->nu;   // rows restricted along x
-  residual<KT, NT>(B, s, r);
+  if (!left) residual<KT, NT>(B, s, r);
   __syncthreads();
   const int n1c = (L.nx >> 1) + 1;
   const T w0 = L.w0, w1 = L.w1, w2 = L.w2;
@@ -548,8 +569,8 @@ template <class KT, int NT, class T>
 __device__ __forceinline__ void level_step(Blk<T>& B, const ClStep& st) {
   const Slab<T> s(B, st.level);
   if (st.op == CL_JACOBI) jacobi<KT, NT>(B, s, st.arg);
-  else if (st.op == CL_GMRES) gmres<KT, NT>(B, s, st.arg, st.zero != 0);
-  else restrict_to<KT, NT>(B, s, st.level);
+  else if (st.op == CL_GMRES) gmres<KT, NT>(B, s, st.arg, st.zero != 0, st.left != 0);
+  else restrict_to<KT, NT>(B, s, st.level, st.left != 0);
 }
 
 template <class T, int NT> __device__ __forceinline__ void cluster_cycle(const ClArgs<T>& a, int rhs, cx<T>* smem) {
@@ -682,26 +703,48 @@ template <class T> cudaError_t launch(bool rag, void* arg, int C, int n, size_t 
 
 }  // namespace
 
-template <class T> int cluster_size(int B) {
-  if (configure<T>(false) != cudaSuccess || configure<T>(true) != cudaSuccess) return 0;
-  for (int C = CL_MAXC; C > 1; C >>= 1) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)C);
-    cfg.blockDim = dim3(cl_threads<T>());
-    cfg.dynamicSmemBytes = CL_SMEM;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern<T>(false), &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
+// Clusters of 2, 4, .. CL_MAXC blocks that the current device runs at once,
+// and the kernels' attributes on it: a property of the device, asked for once
+// (the queries take about half a millisecond, a tenth of a setup).
+template <class T> static const int* cluster_counts() {
+  constexpr int MAXDEV = 64, NC = 5;
+  static_assert(1 << (NC - 1) == CL_MAXC, "cluster sizes");
+  static std::mutex mu;
+  static int table[MAXDEV][NC];   // [k]: clusters of 2^k blocks
+  static bool known[MAXDEV];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAXDEV) return nullptr;
+  std::lock_guard<std::mutex> lk(mu);
+  if (!known[dev]) {
+    if (configure<T>(false) != cudaSuccess || configure<T>(true) != cudaSuccess) return nullptr;
+    for (int k = 1; k < NC; ++k) {
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(1u << k);
+      cfg.blockDim = dim3(cl_threads<T>());
+      cfg.dynamicSmemBytes = CL_SMEM;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = 1u << k;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, kern<T>(false), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+      table[dev][k] = n;
     }
-    if (n >= B) return C;
+    known[dev] = true;
   }
+  return table[dev];
+}
+
+template <class T> int cluster_size(int B) {
+  const int* n = cluster_counts<T>();
+  if (!n) return 0;
+  for (int k = 4; k >= 1; --k)
+    if (n[k] >= B) return 1 << k;
   return 1;
 }
 
@@ -745,7 +788,7 @@ template <class T> bool cluster_layout(std::vector<ClLev<T>>& lv, int C, bool gm
   nX = std::max((nX + al - 1) / al * al, (long long)(((size_t)N * sizeof(double2) / 2 + sizeof(cx<T>)) / sizeof(cx<T>) + al) / al * al);
   a.nu = (int)nu;
   a.nX = (int)nX;
-  a.ou = take(nu * (gmres ? (sizeof(T) == 8 ? 4 : 3) : 2));
+  a.ou = take(nu * (gmres ? 4 : 2));
   a.oX = take(2 * nX);
   a.ored = take(reals((long long)CL_NV * (2 * C + 1 + cl_threads<T>() / 32) + GS));
   a.olev = take((long long)(sizeof(ClLev<T>) * nl + sizeof(cx<T>) - 1) / (long long)sizeof(cx<T>));

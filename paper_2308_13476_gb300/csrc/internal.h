@@ -262,6 +262,7 @@ constexpr int CL_NV = 16;        // values of a cluster-wide sum
 enum { CL_JACOBI = 0, CL_GMRES = 1, CL_RESTRICT = 2, CL_COARSE = 3, CL_PROLONG = 4 };
 struct ClStep {
   int op, level, arg, zero;   // level: counted from lc; arg: sweeps or steps; zero: x is zero on entry
+  int left;                   // complex64 GMRES: leave the residual in u0; restriction: it is there
 };
 template <class T> struct ClLev {
   int nx, ny, n1, rp;         // intervals, nodes per row, rows per block

@@ -30,6 +30,26 @@ namespace hmg {
 inline double ss_scale(double h, int l) { return 0.25 * h * h * (double)(1ll << (2 * l)); }
 inline double ss_sigma(int kind) { return kind == 1 ? 1.0 : 0.0; }
 
+// Steps between two fresh residuals on the levels whose update forms the next
+// residual by linearity, and whether step `step` of a smoothing call starts
+// from one that the previous update left.
+constexpr int SS_REFRESH = 4;
+__host__ __device__ inline bool ss_carried(int step) { return step % SS_REFRESH != 0; }
+
+// Coefficients of r, v_1, v_2, v_3 in the next residual,
+//   r' = (1 - sigma z_0) r - (z_0 + sigma z_1) v_1 - (z_1 + sigma z_2) v_2 - z_2 v_3,
+// from y = scale z.
+__device__ __forceinline__ void ss_residual_coef(const float2 (&y)[3], float iscale, float sigma, float2 (&c)[4]) {
+  float2 z[4];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) z[k] = make_float2(y[k].x * iscale, y[k].y * iscale);
+  z[3] = make_float2(0.f, 0.f);
+  c[0] = make_float2(1.f - sigma * z[0].x, -sigma * z[0].y);
+#pragma unroll
+  for (int k = 1; k < 4; ++k)
+    c[k] = make_float2(-fmaf(sigma, z[k].x, z[k - 1].x), -fmaf(sigma, z[k].y, z[k - 1].y));
+}
+
 // Values of one Gram sum: |v_0|^2 .. |v_3|^2, then <v_i, v_j> (re, im) for
 // (i, j) = (0,1), (0,2), (0,3), (1,2), (1,3), (2,3).
 constexpr int SS_NV = 16;

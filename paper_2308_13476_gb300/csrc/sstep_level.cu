@@ -24,8 +24,6 @@
 namespace hmg {
 namespace {
 
-constexpr int SS_REFRESH = 4;   // steps between two fresh residuals
-
 // What one application forms: RES b - A v, NEXT B v, GRAM v3 = B v2 with the
 // Gram sums and the solve.
 enum { RES = 0, NEXT = 1, GRAM = 2 };
@@ -344,16 +342,7 @@ __device__ __forceinline__ void sl_update_body(const SuA& a, uint3 blk, int rhs)
   float2 y[3], c[4];
 #pragma unroll
   for (int k = 0; k < 3; ++k) y[k] = make_float2(S[2 * k], S[2 * k + 1]);
-  if constexpr (NR) {   // r' = (1 - sigma z0) r - (z0 + sigma z1) v1 - (z1 + sigma z2) v2 - z2 v3, z = y / scale
-    float2 z[4];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) z[k] = make_float2(y[k].x * a.iscale, y[k].y * a.iscale);
-    z[3] = make_float2(0.f, 0.f);
-    c[0] = make_float2(1.f - a.sigma * z[0].x, -a.sigma * z[0].y);
-#pragma unroll
-    for (int k = 1; k < 4; ++k)
-      c[k] = make_float2(-fmaf(a.sigma, z[k].x, z[k - 1].x), -fmaf(a.sigma, z[k].y, z[k - 1].y));
-  }
+  if constexpr (NR) ss_residual_coef(y, a.iscale, a.sigma, c);
   for (int q = 0, j = blk.y * BY * g.ry + threadIdx.y; q < g.ry; ++q, j += BY) {
     if (j > g.ny) break;
     const long long p = off + g.at(i0, j);
@@ -417,9 +406,6 @@ void launch_update(const SuA& a, int B, bool z, bool nr, bool out, cudaStream_t 
   }
 }
 
-// Whether step `step` of nu starts from a residual the previous update left.
-bool carried(int step) { return step % SS_REFRESH != 0; }
-
 }  // namespace
 
 long long sl_blocks(const Grid& g) { return (long long)cdiv(g.nx + 1, BX) * cdiv(g.ny + 1, BY); }
@@ -437,10 +423,10 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
     const float2* r = u0;
     for (int step = 0; step < nu; ++step) {
       const bool z = step == 0 && gb.x_zero, last = step == nu - 1;
-      const bool nr = last ? want_r : carried(step + 1), out = last && gb.outer;
+      const bool nr = last ? want_r : ss_carried(step + 1), out = last && gb.outer;
       if (z) {
         r = b;
-      } else if (!carried(step)) {
+      } else if (!ss_carried(step)) {
         apply(std::integral_constant<int, RES>{}, x, u0);
         r = u0;
       }
@@ -536,8 +522,8 @@ void gmres_smooth_ss_rag(const std::vector<RagLevel<float>>& v, int nu, bool wan
     };
     auto buf = [](int k) { return [k](const RagLevel<float>& L) { return (float2*)(k < 3 ? L.gb.u[k] : L.gb.w); }; };
     for (int step = 0; step < nu; ++step) {
-      const bool nr = step == nu - 1 ? want_r : carried(step + 1);
-      if (!carried(step)) apply(std::integral_constant<int, RES>{}, [](const RagLevel<float>& L) { return L.x; }, buf(0));
+      const bool nr = step == nu - 1 ? want_r : ss_carried(step + 1);
+      if (!ss_carried(step)) apply(std::integral_constant<int, RES>{}, [](const RagLevel<float>& L) { return L.x; }, buf(0));
       apply(std::integral_constant<int, NEXT>{}, buf(0), buf(1));
       apply(std::integral_constant<int, NEXT>{}, buf(1), buf(2));
       apply(std::integral_constant<int, GRAM>{}, buf(2), [&](const RagLevel<float>& L) { return nr ? (float2*)L.gb.w : nullptr; });
