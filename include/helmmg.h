@@ -102,11 +102,9 @@ typedef struct {
                        restriction (needs fuse = 1): 1 = always, 0 = never (the
                        node-parallel kernels; same results to rounding),
                        -1 = the Kronecker-form levels and the complex64 fine
-                       level always, the complex128 fine level when it holds
-                       at least 4 M nodes over all right-hand sides and the
-                       other problems of a ragged batch (its row march keeps
-                       each warp on one strip, which needs that much work to
-                       fill the GPU)                                         */
+                       level; the complex128 fine level runs node-parallel
+                       (the FP64 pipe bounds it, and the marches' halos cost
+                       more there than the passes that they save)            */
   int krylov;       /* 0 = the stand-alone cycle iteration (the paper's method);
                        m in 1..32 = restarted flexible GMRES(m) on the fine
                        operator with one cycle (from zero) as the right
@@ -280,12 +278,14 @@ mg_status mg_two_grid(mg_handle h, int nu, int max_iter, double* out);
 /* Time one kernel of the hierarchy in the handle's precision: `what` = 0 one
  * weighted-Jacobi sweep, 1 a residual b - A x, 2 a restriction, 3 a
  * prolongation-and-correct, 4 one GMRES(3) smoothing step (Sec. 5.3; the
- * kernels the cycle runs for that level: on level 0, when it runs as row
- * marches (option march), four row-march passes and the update, 16 vector
- * reads and writes per node (complex64: three passes and the update, 13, the
- * last Arnoldi vector's norm coming from the Gram form); on a Kronecker-form
- * level with column marches in complex64, five passes with two of them
- * fused, 19; otherwise eight passes, 28 (complex64: seven, 23); needs
+ * kernels the cycle runs for that level, with *bytes counted for the Arnoldi
+ * form of the step: on level 0, when it runs as row marches (option march),
+ * four row-march passes and the update, 16 vector reads and writes per node
+ * (complex64: 13, the last Arnoldi vector's norm coming from the Gram form);
+ * on a Kronecker-form level with column marches in complex64, five passes
+ * with two of them fused, 19; otherwise eight passes, 28 (complex64: seven,
+ * 23); the s-step form that the complex64 levels run moves less: 5 on level
+ * 0, at most 15 on a level that stores its Krylov vectors; needs
  * smoother = 1), 5 the last Arnoldi step of an FGMRES(m) restart cycle
  * (j = m - 1: the pass for the m MGS coefficients and the pass for the new
  * basis vector, which also writes the cycle's right-hand side and zeroes its

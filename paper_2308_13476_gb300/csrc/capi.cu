@@ -80,7 +80,6 @@ struct Level {
 
 struct mg_ctx {
   mg_options opt;
-  long long peer_nodes = 0;   // ragged sub-handle: fine-level nodes of the problems solved beside it
   int nx = 0, ny = 0, B = 1, nlev = 0, ncoarse = 0;
   double h = 0, kconst = 0, beta2 = 0;
   Xfer xw = xfer_of(0);   // inter-grid transfer weights (opt.transfer)
@@ -268,20 +267,16 @@ template <class T> static cudaError_t alloc_vectors(mg_ctx* c, LevelVec<T>& v, c
 
 // ----------------------------------------------------------------- cycle emission
 
-// nu GMRES(3) smoothing steps on level l: the fine level as row marches, the
-// Kronecker-form levels with column-march operator kernels (both with
-// fuse = 1), stored stencils (or fuse = 0) with the node-parallel kernels.
 // Whether level l runs its GMRES(3) kernels as marches (option march).
-// Automatic: the Kronecker-form levels always (their column marches cut the
-// arithmetic of every apply); the fine level when it holds at least 4 M nodes
-// over all right-hand sides, counting those of the other problems of a
-// ragged batch, which run beside it (a row march keeps each warp on one
-// strip, and less work leaves the GPU under-filled).
+// Automatic: the Kronecker-form levels (their column marches cut the
+// arithmetic of every apply).  The complex128 fine level is bound by the FP64
+// pipe, on which the row marches' halo rows and columns cost more than the
+// passes over memory that they save; a step, row marches against
+// node-parallel: 8 x 513^2 1120 / 847 us, 3 x 1025^2 1628 / 1110, 24 x 1025^2
+// 9577 / 7672, 2 x 2049^2 3518 / 2599.
 static bool use_march(const mg_ctx* c, int l) {
   if (!c->opt.fuse || c->opt.march == 0) return false;
-  if (c->opt.march == 1 || c->lev[l].kind >= 4) return true;
-  const Grid& g = c->lev[l].g;
-  return (long long)(g.nx + 1) * (g.ny + 1) * c->B + c->peer_nodes >= (4LL << 20);
+  return c->opt.march == 1 || c->lev[l].kind >= 4;
 }
 
 // Whether level l's complex64 GMRES(3) steps run as the s-step row marches:
@@ -1355,19 +1350,6 @@ mg_status mg_setup_ragged(mg_handle* out, int nprob, const int* nx, const int* n
       FAIL(MG_ENOMEM, "ragged batch: staging buffers of problem %d's group", p);
     }
     c->stage.push_back(stg);
-  }
-  long long total = 0;
-  for (mg_ctx* q : c->sub) total += (long long)(q->nx + 1) * (q->ny + 1) * q->B;
-  // The fine-level kernels (use_march) are chosen for the whole batch's
-  // load, except on the largest problems: they run the most cycles, their
-  // chain of cycles is the batch's critical path, and they decide by their
-  // own size (a single large right-hand side runs its fine level faster
-  // node-parallel than as row marches).
-  long long nmax = 0;
-  for (mg_ctx* q : c->sub) nmax = std::max(nmax, (long long)(q->nx + 1) * (q->ny + 1));
-  for (mg_ctx* q : c->sub) {
-    const long long own = (long long)(q->nx + 1) * (q->ny + 1);
-    q->peer_nodes = own == nmax ? 0 : total - own * q->B;
   }
   c->nx = c->sub[0]->nx;
   c->ny = c->sub[0]->ny;
