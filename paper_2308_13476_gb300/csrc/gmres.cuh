@@ -1,5 +1,5 @@
 // Scalar part of the GMRES(3) smoother (Sec. 5.3 of the paper), shared by
-// the grid-wide kernels and the single-CTA coarse-cycle interpreter: the
+// the grid-wide kernels, the coarse-cycle cluster and the cooperative interpreter: the
 // per-RHS state layout, the Hessenberg updates of one Arnoldi step (modified
 // Gram-Schmidt written with the Gram matrix of the basis) and the FP64 Givens
 // least-squares solve.  Each function runs in one thread.

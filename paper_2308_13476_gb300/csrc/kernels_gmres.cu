@@ -35,7 +35,6 @@ struct GbA {
   double* partial;
   unsigned* tickets;
   const int* active;
-  int ws;
 };
 
 template <class T>
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(BX * BY) g_arn_a(Grid g, Op op, const cx<T>* _
 
 // u_{J+1} = w - sum_{i<=J} h_iJ s_i u_i ; partials |u_{J+1}|^2 and <u_{J+1}, u_l>, l <= J (J < 2)
 template <class T, int J>
-__device__ __forceinline__ void g_arn_b_body(uint3 vblk, dim3 vgrid, Grid g, const cx<T>* __restrict__ u0, const cx<T>* __restrict__ u1, const cx<T>* __restrict__ u2, cx<T>* __restrict__ un, const cx<T>* __restrict__ w, double* __restrict__ st, double* partial, unsigned* tickets, const int* __restrict__ active, int ws) {
+__device__ __forceinline__ void g_arn_b_body(uint3 vblk, dim3 vgrid, Grid g, const cx<T>* __restrict__ u0, const cx<T>* __restrict__ u1, const cx<T>* __restrict__ u2, cx<T>* __restrict__ un, const cx<T>* __restrict__ w, double* __restrict__ st, double* partial, unsigned* tickets, const int* __restrict__ active) {
   const uint3 blockIdx = vblk;   // the block and grid inside this problem's launch
   const dim3 gridDim = vgrid;
   (void)blockIdx;
@@ -173,16 +172,10 @@ __device__ __forceinline__ void g_arn_b_body(uint3 vblk, dim3 vgrid, Grid g, con
       const T sl = S[G_S + l];
       c[l] = mk<T>((T)(hr * sl), (T)(hi * sl));
     }
-    // ws >= 0: w was stored without its scale s_ws (fused Kronecker marches)
-    const T wsc = ws >= 0 ? (T)S[G_S + ws] : T(1);
     GROWS {
       if (j > g.ny) break;
       const int p = g.at(i0, j);
       Pack<T> a = load_pack(w + off, p);
-      if (ws >= 0) {
-#pragma unroll
-        for (int n = 0; n < NP; ++n) a.v[n] = scl<T>(wsc, a.v[n]);
-      }
       Pack<T> uu[J + 1];
 #pragma unroll
       for (int l = 0; l <= J; ++l) {
@@ -208,8 +201,8 @@ __device__ __forceinline__ void g_arn_b_body(uint3 vblk, dim3 vgrid, Grid g, con
 }
 
 template <class T, int J>
-__global__ void __launch_bounds__(BX * BY) g_arn_b(Grid g, const cx<T>* __restrict__ u0, const cx<T>* __restrict__ u1, const cx<T>* __restrict__ u2, cx<T>* __restrict__ un, const cx<T>* __restrict__ w, double* __restrict__ st, double* partial, unsigned* tickets, const int* __restrict__ active, int ws) {
-  g_arn_b_body<T, J>(blockIdx, gridDim, g, u0, u1, u2, un, w, st, partial, tickets, active, ws);
+__global__ void __launch_bounds__(BX * BY) g_arn_b(Grid g, const cx<T>* __restrict__ u0, const cx<T>* __restrict__ u1, const cx<T>* __restrict__ u2, cx<T>* __restrict__ un, const cx<T>* __restrict__ w, double* __restrict__ st, double* partial, unsigned* tickets, const int* __restrict__ active) {
+  g_arn_b_body<T, J>(blockIdx, gridDim, g, u0, u1, u2, un, w, st, partial, tickets, active);
 }
 
 template <class T, int J>
@@ -217,7 +210,7 @@ __global__ void __launch_bounds__(BX * BY) g_arn_b_rag(const __grid_constant__ R
   uint3 vb;
   dim3 vg;
   const GbA<T>& a = L.a[rag_problem(L, blockIdx.x, vb, vg)];
-  g_arn_b_body<T, J>(vb, vg, a.g, a.u0, a.u1, a.u2, a.un, a.w, a.st, a.partial, a.tickets, a.active, a.ws);
+  g_arn_b_body<T, J>(vb, vg, a.g, a.u0, a.u1, a.u2, a.un, a.w, a.st, a.partial, a.tickets, a.active);
 }
 
 // x += sum_{i<m} y_i s_i u_i
@@ -294,11 +287,11 @@ void gmres_smooth(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<T>* b,
       if (z) g_init_zero<T><<<grd, blk, 0, s>>>(g, b, st, P, tk, active);
       else g_init<T, Op><<<grd, blk, 0, s>>>(g, op, x, b, u0, st, P, tk, active);
       g_arn_a<T, Op, 0><<<grd, blk, 0, s>>>(g, op, v0, u1, u2, w, st, P, tk, active);
-      g_arn_b<T, 0><<<grd, blk, 0, s>>>(g, v0, u1, u2, u1, w, st, P, tk, active, -1);
+      g_arn_b<T, 0><<<grd, blk, 0, s>>>(g, v0, u1, u2, u1, w, st, P, tk, active);
       g_arn_a<T, Op, 1><<<grd, blk, 0, s>>>(g, op, v0, u1, u2, w, st, P, tk, active);
-      g_arn_b<T, 1><<<grd, blk, 0, s>>>(g, v0, u1, u2, u2, w, st, P, tk, active, -1);
+      g_arn_b<T, 1><<<grd, blk, 0, s>>>(g, v0, u1, u2, u2, w, st, P, tk, active);
       g_arn_a<T, Op, 2><<<grd, blk, 0, s>>>(g, op, v0, u1, u2, w, st, P, tk, active);
-      g_arn_b<T, 2><<<grd, blk, 0, s>>>(g, v0, u1, u2, nullptr, w, st, P, tk, active, -1);
+      g_arn_b<T, 2><<<grd, blk, 0, s>>>(g, v0, u1, u2, nullptr, w, st, P, tk, active);
       GmresBufs gs = gb;
       gs.u[0] = (void*)v0;
       g_update<T><<<grd, blk, 0, s>>>(g, x, v0, u1, u2, st, active);
@@ -315,10 +308,10 @@ void launch_gmres_update(const Grid& g, cx<T>* x, const GmresBufs& gb, int B, co
 }
 
 template <class T, int J>
-void launch_arn_b(const Grid& g, const GmresBufs& gb, cx<T>* un, int B, const int* active, cudaStream_t s, int ws) {
+void launch_arn_b(const Grid& g, const GmresBufs& gb, cx<T>* un, int B, const int* active, cudaStream_t s) {
   dim3 grd(cdiv(g.nx + 1, BX * PK<T>::NP), cdiv(g.ny + 1, BY * g.ry), B);
   g_arn_b<T, J><<<grd, dim3(BX, BY), 0, s>>>(g, (const cx<T>*)gb.u[0], (const cx<T>*)gb.u[1], (const cx<T>*)gb.u[2],
-                                            un, (const cx<T>*)gb.w, gb.st, gb.partial, gb.tickets, active, ws);
+                                            un, (const cx<T>*)gb.w, gb.st, gb.partial, gb.tickets, active);
 }
 
 template <class T> void launch_gmres_update_rag(const std::vector<RagLevel<T>>& v, cudaStream_t s) {
@@ -332,12 +325,12 @@ template <class T> void launch_gmres_update_rag(const std::vector<RagLevel<T>>& 
 }
 
 template <class T, int J>
-void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next, int ws, cudaStream_t s) {
+void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next, cudaStream_t s) {
   rag_launch<GbA<T>>((int)v.size(), g_arn_b_rag<T, J>, dim3(BX, BY), 0, s, [&](int q, GbA<T>& a, int& gx, int& gy) {
     const RagLevel<T>& L = v[q];
     cx<T>* un = un_next && J < 2 ? (cx<T>*)L.gb.u[J + 1] : nullptr;
     a = GbA<T>{L.g, (const cx<T>*)L.gb.u[0], (const cx<T>*)L.gb.u[1], (const cx<T>*)L.gb.u[2], un,
-               (const cx<T>*)L.gb.w, L.gb.st, L.gb.partial, L.gb.tickets, L.active, ws};
+               (const cx<T>*)L.gb.w, L.gb.st, L.gb.partial, L.gb.tickets, L.active};
     gx = cdiv(L.g.nx + 1, BX * PK<T>::NP);
     gy = cdiv(L.g.ny + 1, BY * L.g.ry);
     return true;
@@ -345,12 +338,12 @@ void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next, int ws, c
 }
 
 template void launch_gmres_update_rag<double>(const std::vector<RagLevel<double>>&, cudaStream_t);
-template void launch_arn_b_rag<double, 0>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
-template void launch_arn_b_rag<double, 1>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
-template void launch_arn_b_rag<double, 2>(const std::vector<RagLevel<double>>&, bool, int, cudaStream_t);
-template void launch_arn_b<double, 0>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
-template void launch_arn_b<double, 1>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
-template void launch_arn_b<double, 2>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t, int);
+template void launch_arn_b_rag<double, 0>(const std::vector<RagLevel<double>>&, bool, cudaStream_t);
+template void launch_arn_b_rag<double, 1>(const std::vector<RagLevel<double>>&, bool, cudaStream_t);
+template void launch_arn_b_rag<double, 2>(const std::vector<RagLevel<double>>&, bool, cudaStream_t);
+template void launch_arn_b<double, 0>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t);
+template void launch_arn_b<double, 1>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t);
+template void launch_arn_b<double, 2>(const Grid&, const GmresBufs&, double2*, int, const int*, cudaStream_t);
 template void launch_gmres_update<double>(const Grid&, double2*, const GmresBufs&, int, const int*, cudaStream_t);
 template void gmres_smooth<double>(const Grid&, const OpView<double>&, double2*, const double2*, int, int, const int*,
                                    const GmresBufs&, cudaStream_t);

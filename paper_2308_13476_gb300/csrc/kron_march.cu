@@ -203,7 +203,7 @@ template <class T, int R> long long kron_capacity() {
 template <class T> void launch_gmres_update(const Grid& g, cx<T>* x, const GmresBufs& gb, int B, const int* active,
                                             cudaStream_t s);
 template <class T, int J> void launch_arn_b(const Grid& g, const GmresBufs& gb, cx<T>* un, int B, const int* active,
-                                            cudaStream_t s, int ws);
+                                            cudaStream_t s);
 
 long long kron_march_blocks(const Grid& g, int B) {   // the most for any chunk height: the shortest
   (void)B;
@@ -233,11 +233,11 @@ void gmres_smooth_kron(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<T
       if (z) km_init_zero<T><<<grd, KW * 32, 0, s>>>(g, kg, b, st, P, tk, active);
       else km_init<T, R><<<grd, KW * 32, 0, s>>>(g, kg, op, x, b, u0, st, P, tk, active);
       km_arn_a<T, R, 0><<<grd, KW * 32, 0, s>>>(g, kg, op, v0, u1, u2, w, st, P, tk, active);
-      launch_arn_b<T, 0>(g, gs, u1, B, active, s, -1);
+      launch_arn_b<T, 0>(g, gs, u1, B, active, s);
       km_arn_a<T, R, 1><<<grd, KW * 32, 0, s>>>(g, kg, op, v0, u1, u2, w, st, P, tk, active);
-      launch_arn_b<T, 1>(g, gs, u2, B, active, s, -1);
+      launch_arn_b<T, 1>(g, gs, u2, B, active, s);
       km_arn_a<T, R, 2><<<grd, KW * 32, 0, s>>>(g, kg, op, v0, u1, u2, w, st, P, tk, active);
-      launch_arn_b<T, 2>(g, gs, nullptr, B, active, s, -1);
+      launch_arn_b<T, 2>(g, gs, nullptr, B, active, s);
       launch_gmres_update<T>(g, x, gs, B, active, s);
     }
   };
@@ -301,11 +301,11 @@ void gmres_smooth_kron_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream
     for (int step = 0; step < nu; ++step) {
       launch(km_init_rag<T, R>, none);
       launch(km_arn_a_rag<T, R, 0>, none);
-      launch_arn_b_rag<T, 0>(v, true, -1, s);
+      launch_arn_b_rag<T, 0>(v, true, s);
       launch(km_arn_a_rag<T, R, 1>, none);
-      launch_arn_b_rag<T, 1>(v, true, -1, s);
+      launch_arn_b_rag<T, 1>(v, true, s);
       launch(km_arn_a_rag<T, R, 2>, none);
-      launch_arn_b_rag<T, 2>(v, false, -1, s);
+      launch_arn_b_rag<T, 2>(v, false, s);
       launch_gmres_update_rag<T>(v, s);
     }
   };

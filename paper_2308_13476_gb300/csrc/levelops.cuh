@@ -1,5 +1,4 @@
-// Device helpers shared by the coarse-cycle interpreters (coarse.cu and
-// coop.cu): operator apply and inverse diagonal of a level described by a
+// Device helpers of the cooperative coarse-cycle interpreter (coop.cu): operator apply and inverse diagonal of a level described by a
 // CLevel.
 #pragma once
 #include "internal.h"

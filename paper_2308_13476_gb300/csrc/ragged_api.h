@@ -30,8 +30,8 @@ template <class T> void gmres_smooth_march_rag(const std::vector<RagLevel<T>>& v
                                                cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 template <class T> void gmres_smooth_kron_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream_t s);
 template <class T> void launch_gmres_update_rag(const std::vector<RagLevel<T>>& v, cudaStream_t s);
-// g_arn_b<J> on every problem; un_next: store u_{J+1} (into u[J+1]); ws as g_arn_b
-template <class T, int J> void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next, int ws,
+// g_arn_b<J> on every problem; un_next: store u_{J+1} (into u[J+1])
+template <class T, int J> void launch_arn_b_rag(const std::vector<RagLevel<T>>& v, bool un_next,
                                                 cudaStream_t s);
 
 // One problem's inter-grid transfer between level l (fine) and l + 1.
