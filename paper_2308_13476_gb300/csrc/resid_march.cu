@@ -91,6 +91,8 @@ struct CSum {
     lo += (hi - (s - z)) + (t - z);
     hi = s;
   }
+  // past the largest float lo is inf - inf: the sum is then hi, inf
+  __device__ __forceinline__ float total() const { return lo == lo ? hi + lo : hi; }
 };
 
 template <bool VK> struct RmMarch {
@@ -226,7 +228,7 @@ template <bool A2, bool VK> __device__ __forceinline__ void rm_body(const RmA& a
       sum.add(fmaf(f.x, f.x, f.y * f.y));
     }
   }
-  const float a0[1] = {sum.hi + sum.lo};
+  const float a0[1] = {sum.total()};
   double v[1];
   __syncwarp();
   if (reduce_last<1, float>(a0, v, sh, a.c.partial, a.c.tickets, rhs, a.m.blocks(), blk) && threadIdx.x == 0)
