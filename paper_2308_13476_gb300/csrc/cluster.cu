@@ -150,10 +150,10 @@ __device__ __forceinline__ void cl_push_sum(Blk<T>& B, T (&v)[NV]) {
       for (int w = 1; w < W; ++w) s += B.wsum[lane * W + w];
     }
     T* mine = B.red + (B.rpar * B.C + B.rank) * CL_NV;
-    for (int e = lane; e < NV * B.C; e += 32) {   // NV divides 32 or is 32 / 2^k: the value stays in range
-      const int k = e % NV;
-      const T sv = __shfl_sync(__activemask(), s, k);
-      cl_st(cl_map(mine + k, e / NV), sv);
+    for (int e0 = 0; e0 < NV * B.C; e0 += 32) {   // the whole warp takes part in every exchange
+      const int e = e0 + lane, k = e % NV;
+      const T sv = __shfl_sync(0xffffffffu, s, k);
+      if (e < NV * B.C) cl_st(cl_map(mine + k, e / NV), sv);
     }
   }
 }
