@@ -103,6 +103,7 @@ struct mg_ctx {
   int* state = nullptr;
   int* cycles = nullptr;
   double* relres = nullptr;
+  float* rscale = nullptr;   // mixed: [B][2], Ctl::rscale
   double* hist = nullptr;
   int hist_len = 0;
   double* bnorm = nullptr;
@@ -261,6 +262,7 @@ template <class T> static cudaError_t alloc_vectors(mg_ctx* c, LevelVec<T>& v, c
     v.gb.partial = c->partial;
     v.gb.tickets = c->tickets;
     v.gb.st = c->gst;
+    v.gb.rscale = c->rscale;
   }
   return cudaSuccess;
 }
@@ -432,7 +434,7 @@ template <class T> struct Emit {
 
 static Ctl ctl(const mg_ctx* c) {
   return Ctl{c->bnorm, c->tolp, c->active, c->state, c->cycles, c->relres, c->hist, c->hist_len, c->n_active,
-             c->partial, c->tickets};
+             c->partial, c->tickets, c->rscale};
 }
 
 // Records the steps of one visit of level lc (the same recursion as
@@ -639,11 +641,11 @@ static void emit_mixed_iteration(mg_ctx* c, cudaStream_t s) {
   e.zx[0] = 1;
   e.cycle(0);
   if (c->opt.precision == 2) {
-    launch_ff_update(g0, c->v64[0].x, e.cur[0], c->B, c->active, s);
+    launch_ff_update(g0, c->v64[0].x, e.cur[0], c->B, c->active, c->rscale, s);
     launch_ff_resid_cast_stop(g0, c->hffc, c->kf64, c->h, c->ffdiag, c->v64[0].x, c->v64[0].b, c->v32[0].b, c->B,
                               ctl(c), 1, s);
   } else {
-    if (!fused) launch_update_mixed(g0, c->v64[0].x, e.cur[0], c->B, c->active, s);
+    if (!fused) launch_update_mixed(g0, c->v64[0].x, e.cur[0], c->B, c->active, c->rscale, s);
     launch_resid_cast_stop(g0, op64(c, 0), c->v64[0].x, c->v64[0].b, c->v32[0].b, c->B, ctl(c), 1, s);
   }
 }
@@ -659,6 +661,7 @@ static FgArgs fg_args(const mg_ctx* c, double tol) {
   a.state = c->state;
   a.cycles = c->cycles;
   a.relres = c->relres;
+  a.rscale = c->rscale;
   a.hist = c->hist;
   a.hist_len = c->hist_len;
   a.n_active = c->n_active;
@@ -1146,6 +1149,11 @@ static mg_status setup_impl(mg_ctx* c, const double* k_field) {
   CK(dalloc(c, (void**)&c->state, sizeof(int) * c->B));
   CK(dalloc(c, (void**)&c->cycles, sizeof(int) * c->B));
   CK(dalloc(c, (void**)&c->relres, sizeof(double) * c->B));
+  if (mixed) {
+    const std::vector<float> one(2 * c->B, 1.f);
+    CK(dalloc(c, (void**)&c->rscale, sizeof(float) * 2 * c->B));
+    CK(cudaMemcpyAsync(c->rscale, one.data(), sizeof(float) * 2 * c->B, cudaMemcpyHostToDevice, s));
+  }
   CK(dalloc(c, (void**)&c->bnorm, sizeof(double) * c->B));
   CK(dalloc(c, (void**)&c->tolp, sizeof(double) * 2));
   CK(dalloc(c, (void**)&c->n_active, sizeof(int) * 2));   // {active count, cooperative-barrier error}
@@ -1449,7 +1457,7 @@ static mg_status solve_fgmres(mg_ctx* c, const void* rhs, void* x, double tol, i
   const FgArgs a = fg_args(c, tol);
   launch_pack<double>(g0, (const double2*)rhs, (double2*)a.b, B, conj, s);
   launch_pack<double>(g0, (const double2*)x, a.X, B, conj, s);
-  launch_vecnorm_fin<double>(g0, a.b, B, c->bnorm, c->partial, c->tickets, s);
+  launch_vecnorm_fin<double>(g0, a.b, B, c->bnorm, c->partial, c->tickets, s, c->rscale);
   std::vector<double> bn(B);
   CK(cudaMemcpyAsync(bn.data(), c->bnorm, sizeof(double) * B, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
@@ -1543,11 +1551,11 @@ static mg_status solve_begin(mg_ctx* c, const void* rhs, void* x, double tol, in
   if (ffo) {   // level-0 outer vectors in float-float
     launch_ff_pack(g0, (const double2*)rhs, c->v64[0].b, B, conj, s);
     launch_ff_pack(g0, (const double2*)x, c->v64[0].x, B, conj, s);
-    launch_ff_norm(g0, c->v64[0].b, B, c->bnorm, c->partial, c->tickets, s);
+    launch_ff_norm(g0, c->v64[0].b, B, c->bnorm, c->partial, c->tickets, c->rscale, s);
   } else {
     launch_pack<double>(g0, (const double2*)rhs, c->v64[0].b, B, conj, s);
     launch_pack<double>(g0, (const double2*)x, c->v64[0].x, B, conj, s);
-    launch_vecnorm_fin<double>(g0, c->v64[0].b, B, c->bnorm, c->partial, c->tickets, s);
+    launch_vecnorm_fin<double>(g0, c->v64[0].b, B, c->bnorm, c->partial, c->tickets, s, c->rscale);
   }
   std::vector<double> bn(B);
   CK(cudaMemcpyAsync(bn.data(), c->bnorm, sizeof(double) * B, cudaMemcpyDeviceToHost, s));

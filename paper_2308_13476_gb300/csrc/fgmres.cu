@@ -149,6 +149,8 @@ __global__ void __launch_bounds__(FTHREADS) k_fg_restart(FgArgs a, cx<T>* __rest
   const double2* x = a.X + off;
   const double2* b = a.b + off;
   cx<T>* v0 = (cx<T>*)a.V + off;
+  T gs = T(1);   // complex64: factor of the cycle's right-hand side
+  if constexpr (sizeof(T) == 4) gs = a.rscale[2 * rhs + 1];
   double acc = 0.0;
   for (int s = blockIdx.x; s < a.ns; s += a.nbr) {
     const StripPos sp = strip_pos(a, s);
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(FTHREADS) k_fg_restart(FgArgs a, cx<T>* __rest
       const double2 rr = sub<double>(b[p], op.apply(x, p, g.pitch, sp.i, j));
       const cx<T> u = from_d<T>(rr);
       v0[p] = u;
-      cb[off + p] = u;
+      cb[off + p] = scl<T>(gs, u);
       cxv[off + p] = mk<T>(T(0), T(0));
       acc += abs2<double>(rr);
     }
@@ -194,6 +196,10 @@ __global__ void __launch_bounds__(FTHREADS) k_fg_restart(FgArgs a, cx<T>* __rest
     S[L.g(0)] = beta;
     S[L.beta()] = beta;
     S[L.s(0)] = 1.0 / beta;
+    if constexpr (sizeof(T) == 4) {
+      a.rscale[2 * rhs] = gs;
+      a.rscale[2 * rhs + 1] = inv_pow2(beta);
+    }
     a.active[rhs] = 1;
     atomicAdd(a.n_active, 1);
   }
@@ -258,7 +264,9 @@ __global__ void __launch_bounds__(FTHREADS, FG_MINB<T>) k_fg_dots(FgArgs a, cons
   const cx<T>* zs = z + off;
   cx<T>* zj = (cx<T>*)a.Z + jj * a.vlen + off;
   const cx<T>* vj = (const cx<T>*)a.V + jj * a.vlen + off;
-  const T sj = (T)a.S[(long long)rhs * a.sd + FgLayout{a.m}.s(jj)];   // z_j = s_j M(u_j)
+  double sd = a.S[(long long)rhs * a.sd + FgLayout{a.m}.s(jj)];   // z_j = s_j M(u_j)
+  if constexpr (sizeof(T) == 4) sd *= f64_from_f32(rcp_pow2(a.rscale[2 * rhs]));
+  const T sj = (T)sd;
   for (int s = blockIdx.x; s < a.ns; s += a.nbr) {
     const StripPos sp = strip_pos(a, s);
     cx<T> w[FR], u[FR];
@@ -394,6 +402,7 @@ __device__ void fg_finish_step(const FgArgs& a, int rhs, int jj, double sumsq, i
       atomicSub(a.n_active, 1);
     } else {
       S[L.s(k)] = 1.0 / nrm;
+      if (a.rscale) a.rscale[2 * rhs] = 1.f;   // u_k = A z_{k-1} - .. with z_{k-1} = M(v_{k-1}) is of the size of v
     }
   }
   if (!end) return;

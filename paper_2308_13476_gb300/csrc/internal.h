@@ -87,15 +87,36 @@ struct Ctl {
   int* n_active;        // one int
   double* partial;
   unsigned* tickets;
+  float* rscale;        // complex64 cycles, [B][2] (null: complex128): see inv_pow2
 };
+// The power of two next to 1 / v, of a v that may be 0 or not finite.  A
+// complex64 cycle runs on its right-hand side times such a power of the
+// residual's norm and its result is divided by it again: every step of a cycle
+// is homogeneous, so no digit of the iterates depends on it, and the Gram sums
+// of the s-step smoother (squares of unnormalised vectors) stay in the float
+// range for residuals of any size (with the residual itself, solves that pass
+// below 1e-19 per node took 30 to 60 % more cycles).  rscale[2 rhs] is the
+// factor of the right-hand side at hand, rscale[2 rhs + 1] that of the next one,
+// from the norm before it.
+__device__ __forceinline__ float inv_pow2(double v) {
+  const int e = (int)((unsigned long long)__double_as_longlong(v) >> 52 & 0x7ff) - 1023;
+  return __uint_as_float((unsigned)(127 - max(-126, min(126, e))) << 23);
+}
+// 1 / s of such a power of two: its exponent mirrored
+__device__ __forceinline__ float rcp_pow2(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
 // Stopping test for one right-hand side, run by the last block of a norm
 // reduction: relres = sqrt(sumsq) / ||b||; count != 0 means a cycle has just
 // finished.  A RHS that meets tol (state 1) or diverges (state 2: not finite
 // or above the threshold) is deactivated.
-__device__ __forceinline__ void stop_update(const Ctl& c, int rhs, double sumsq, int count) {
+// gs: the factor that the residual was written with (Ctl::rscale).
+__device__ __forceinline__ void stop_update(const Ctl& c, int rhs, double sumsq, int count, float gs = 1.f) {
   const double tol = c.tolp[0], diverge = c.tolp[1];
-  const double rr = sqrt(sumsq) / c.bnorm[rhs];
+  const double nrm = sqrt(sumsq), rr = nrm / c.bnorm[rhs];
   c.relres[rhs] = rr;
+  if (c.rscale) {
+    c.rscale[2 * rhs] = gs;
+    c.rscale[2 * rhs + 1] = inv_pow2(nrm);
+  }
   if (count) {
     const int cy = ++c.cycles[rhs];
     if (cy <= c.hist_len) c.hist[(long long)rhs * c.hist_len + cy - 1] = rr;
@@ -114,15 +135,17 @@ __device__ __forceinline__ void stop_update(const Ctl& c, int rhs, double sumsq,
 template <class T> void launch_resnorm_stop(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                             int B, const Ctl& c, int count, cudaStream_t s);
 // Mixed path, FP64 outer loop: r = b - A x in FP64, written as float into r32
-// (same Grid), stopping test fused (resid_march.cu; resid_blocks() records per
-// RHS in the partial buffer); and x += e (FP64 += float), masked.
+// (same Grid) times rscale[2 rhs + 1], stopping test fused (resid_march.cu;
+// resid_blocks() records per RHS in the partial buffer); and x += e / rscale[2
+// rhs] (FP64 += float), masked.
 long long resid_blocks(const Grid& g, int B);
 void launch_resid_cast_stop(const Grid& g, const OpView<double>& op, const double2* x, const double2* b,
                             float2* r32, int B, const Ctl& c, int count, cudaStream_t s);
-void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, cudaStream_t s);
-// out[b] = ||v_b|| (one kernel).
+void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, const float* rscale,
+                         cudaStream_t s);
+// out[b] = ||v_b|| (one kernel); rscale: the factors of Ctl::rscale from it.
 template <class T> void launch_vecnorm_fin(const Grid& g, const cx<T>* v, int B, double* out, double* partial,
-                                           unsigned* tickets, cudaStream_t s);
+                                           unsigned* tickets, cudaStream_t s, float* rscale = nullptr);
 // Transfers (weights xw, Eq. (xex) or linear): r_c = R r_f and x_f += P e_c.
 template <class T> void launch_restrict(const Grid& gf, const Grid& gc, const cx<T>* rf, cx<T>* rc, int B,
                                         const int* active, const Xfer& xw, cudaStream_t s);
@@ -183,6 +206,7 @@ struct GmresBufs {
                        // u0 = b - A x (no apply, no u0 write; b is read-only
                        // in every pass) and only sums |b|^2 for its norm
   float scale, sigma;  // complex64 s-step basis of the level (sstep.cuh)
+  const float* rscale; // complex64: Ctl::rscale (the update of outer divides by it)
 };
 template <class T> void gmres_smooth(const Grid& g, const OpView<T>& op, cx<T>* x, const cx<T>* b, int nu, int B,
                                      const int* active, const GmresBufs& gb, cudaStream_t s);
@@ -345,11 +369,12 @@ void launch_ff_resid_cast_stop(const Grid& g, const FFConsts& K, const double* k
                                const void* x, const void* b, float2* r32, int B, const Ctl& c, int count,
                                cudaStream_t s);
 // x += e (float-float += float), masked.
-void launch_ff_update(const Grid& g, void* x, const float2* e, int B, const int* active, cudaStream_t s);
+void launch_ff_update(const Grid& g, void* x, const float2* e, int B, const int* active, const float* rscale,
+                      cudaStream_t s);
 void launch_ff_pack(const Grid& g, const double2* user, void* v, int B, int conj, cudaStream_t s);
 void launch_ff_unpack(const Grid& g, const void* v, double2* user, int B, int conj, cudaStream_t s);
 void launch_ff_norm(const Grid& g, const void* v, int B, double* out, double* partial, unsigned* tickets,
-                    cudaStream_t s);
+                    float* rscale, cudaStream_t s);
 
 // Flexible GMRES(m) outer loop with one cycle as the right preconditioner
 // (fgmres.cu).  V: m+1 basis vectors and Z: m preconditioned vectors, both
@@ -399,6 +424,7 @@ struct FgArgs {
   int max_cycles;
   double* partial;         // [B][nvp][nbr]
   unsigned* tickets;       // [B], 0 at rest
+  float* rscale;           // complex64 cycles: as Ctl::rscale, of the cycle's right-hand side
 };
 // Strip geometry and blocks per RHS (nbr, ncx, ns, nvp) for a fine grid.
 void fg_geometry(const Grid& g, int B, bool fp64z, FgArgs& a);

@@ -46,6 +46,7 @@ struct UmA {
   double2* x;
   const float2* e;
   const int* active;
+  const float* rscale;
 };
 
 template <class T>
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(BX * BY) k_resnorm_stop_rag(const __grid_const
   k_resnorm_stop_body<T, Op>(vb, vg, a.g, a.op, a.x, a.b, a.c, a.count);
 }
 
-__device__ __forceinline__ void k_update_mixed_body(uint3 vblk, dim3 vgrid, Grid g, double2* __restrict__ x, const float2* __restrict__ e, const int* __restrict__ active) {
+__device__ __forceinline__ void k_update_mixed_body(uint3 vblk, dim3 vgrid, Grid g, double2* __restrict__ x, const float2* __restrict__ e, const int* __restrict__ active, const float* __restrict__ rscale) {
   const uint3 blockIdx = vblk;   // the block and grid inside this problem's launch
   const dim3 gridDim = vgrid;
   (void)blockIdx;
@@ -183,32 +184,33 @@ __device__ __forceinline__ void k_update_mixed_body(uint3 vblk, dim3 vgrid, Grid
   NODE_INDEX
   if (active && !active[rhs]) return;
   if (i > g.nx) return;
+  const double ig = f64_from_f32(rcp_pow2(rscale[2 * rhs]));
   FOR_ROWS {
     if (j > g.ny) break;
     const long long p = off + g.at(i, j);
     const float2 d = e[p];
     double2 xv = x[p];
-    xv.x += f64_from_f32(d.x);
-    xv.y += f64_from_f32(d.y);
+    xv.x = fma(ig, f64_from_f32(d.x), xv.x);
+    xv.y = fma(ig, f64_from_f32(d.y), xv.y);
     x[p] = xv;
   }
 }
 
-__global__ void __launch_bounds__(BX * BY) k_update_mixed(Grid g, double2* __restrict__ x, const float2* __restrict__ e, const int* __restrict__ active) {
-  k_update_mixed_body(blockIdx, gridDim, g, x, e, active);
+__global__ void __launch_bounds__(BX * BY) k_update_mixed(Grid g, double2* __restrict__ x, const float2* __restrict__ e, const int* __restrict__ active, const float* __restrict__ rscale) {
+  k_update_mixed_body(blockIdx, gridDim, g, x, e, active, rscale);
 }
 
 __global__ void __launch_bounds__(BX * BY) k_update_mixed_rag(const __grid_constant__ RagLaunch<UmA> L) {
   uint3 vb;
   dim3 vg;
   const UmA& a = L.a[rag_problem(L, blockIdx.x, vb, vg)];
-  k_update_mixed_body(vb, vg, a.g, a.x, a.e, a.active);
+  k_update_mixed_body(vb, vg, a.g, a.x, a.e, a.active, a.rscale);
 }
 
 // ||v|| per RHS into out[rhs] (one kernel, last-block finish).
 template <class T>
 __global__ void __launch_bounds__(BX * BY) k_vecnorm_fin(Grid g, const cx<T>* __restrict__ v_, double* __restrict__ out,
-                                                         double* partial, unsigned* tickets) {
+                                                         double* partial, unsigned* tickets, float* rscale) {
   __shared__ double sh[32];
   NODE_INDEX
   T a0[1] = {T(0)};
@@ -220,8 +222,10 @@ __global__ void __launch_bounds__(BX * BY) k_vecnorm_fin(Grid g, const cx<T>* __
   }
   double v[1];
   if (reduce_last<1, T>(a0, v, sh, partial, tickets, rhs, gridDim.x * gridDim.y, blockIdx.y * gridDim.x + blockIdx.x) &&
-      threadIdx.x == 0 && threadIdx.y == 0)
+      threadIdx.x == 0 && threadIdx.y == 0) {
     out[rhs] = sqrt(v[0]);
+    if (rscale) rscale[2 * rhs] = rscale[2 * rhs + 1] = inv_pow2(out[rhs]);
+  }
 }
 
 // ------------------------------------------------------------------ transfers
@@ -422,13 +426,14 @@ void launch_resnorm_stop(const Grid& g, const OpView<T>& v, const cx<T>* x, cons
     k_resnorm_stop<T, decltype(op)><<<pack_grid(g, B, PK<T>::NP), dim3(BX, BY), 0, s>>>(g, op, x, b, c, count);
   });
 }
-void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, cudaStream_t s) {
-  k_update_mixed<<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, x, e, active);
+void launch_update_mixed(const Grid& g, double2* x, const float2* e, int B, const int* active, const float* rscale,
+                         cudaStream_t s) {
+  k_update_mixed<<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, x, e, active, rscale);
 }
 template <class T>
 void launch_vecnorm_fin(const Grid& g, const cx<T>* v, int B, double* out, double* partial, unsigned* tickets,
-                        cudaStream_t s) {
-  k_vecnorm_fin<T><<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, v, out, partial, tickets);
+                        cudaStream_t s, float* rscale) {
+  k_vecnorm_fin<T><<<node_grid(g, B), dim3(BX, BY), 0, s>>>(g, v, out, partial, tickets, rscale);
 }
 template <class T>
 void launch_restrict(const Grid& gf, const Grid& gc, const cx<T>* rf, cx<T>* rc, int B, const int* active,
@@ -505,7 +510,7 @@ template void launch_prolong_add_rag<float>(const std::vector<RagXfer<float>>&, 
 void launch_update_mixed_rag(const std::vector<RagOuter>& v, cudaStream_t s) {
   rag_launch<UmA>((int)v.size(), k_update_mixed_rag, dim3(BX, BY), 0, s, [&](int q, UmA& a, int& gx, int& gy) {
     const RagOuter& O = v[q];
-    a = UmA{O.g, O.x, O.e, O.c.active};
+    a = UmA{O.g, O.x, O.e, O.c.active, O.c.rscale};
     const dim3 d = node_grid(O.g, 1);
     gx = (int)d.x;
     gy = (int)d.y;
@@ -567,7 +572,8 @@ void launch_gradient(int nx, int ny, double h, const double* m, double omega_f, 
   template void launch_copy_masked<T>(const Grid&, const cx<T>*, cx<T>*, int, const int*, cudaStream_t);          \
   template void launch_pack<T>(const Grid&, const double2*, cx<T>*, int, int, cudaStream_t);                      \
   template void launch_unpack<T>(const Grid&, const cx<T>*, double2*, int, int, cudaStream_t);                    \
-  template void launch_vecnorm_fin<T>(const Grid&, const cx<T>*, int, double*, double*, unsigned*, cudaStream_t);
+  template void launch_vecnorm_fin<T>(const Grid&, const cx<T>*, int, double*, double*, unsigned*, cudaStream_t, \
+                                      float*);
 INST(double)
 INST(float)
 

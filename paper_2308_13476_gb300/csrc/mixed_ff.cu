@@ -107,12 +107,13 @@ __global__ void __launch_bounds__(BX * BY) k_ff_resid_cast_stop(Grid g, FFConsts
   FF_NODE
   if (!c.active[rhs]) return;   // block-uniform
   float a = 0.f;
+  const float gs = c.rscale[2 * rhs + 1];
   if (i <= g.nx) {
     FF_ROWS {
       if (j > g.ny) break;
       const int p = g.at(i, j);
       const cff r = ff_residual(K, kf, g.nx, g.ny, inv_h, dP, x + off, b + off, p, g.pitch, i, j);
-      r32[off + p] = make_float2(r.re.h, r.im.h);
+      r32[off + p] = make_float2(gs * r.re.h, gs * r.im.h);
       a = fmaf(r.re.h, r.re.h, fmaf(r.im.h, r.im.h, a));
     }
   }
@@ -121,21 +122,23 @@ __global__ void __launch_bounds__(BX * BY) k_ff_resid_cast_stop(Grid g, FFConsts
   if (reduce_last<1, double>(ad, v, sh, c.partial, c.tickets, rhs, gridDim.x * gridDim.y,
                              blockIdx.y * gridDim.x + blockIdx.x) &&
       threadIdx.x == 0 && threadIdx.y == 0)
-    stop_update(c, rhs, v[0], count);
+    stop_update(c, rhs, v[0], count, gs);
 }
 
 __global__ void __launch_bounds__(BX * BY) k_ff_update(Grid g, float4* __restrict__ x, const float2* __restrict__ e,
-                                                       const int* __restrict__ active) {
+                                                       const int* __restrict__ active,
+                                                       const float* __restrict__ rscale) {
   FF_NODE
   if (active && !active[rhs]) return;
   if (i > g.nx) return;
+  const float ig = rcp_pow2(rscale[2 * rhs]);
   FF_ROWS {
     if (j > g.ny) break;
     const long long p = off + g.at(i, j);
     const float2 d = e[p];
     cff v = ld(x + p);
-    v.re = ff_add(v.re, {d.x, 0.f});
-    v.im = ff_add(v.im, {d.y, 0.f});
+    v.re = ff_add(v.re, {ig * d.x, 0.f});
+    v.im = ff_add(v.im, {ig * d.y, 0.f});
     st(x + p, v);
   }
 }
@@ -166,7 +169,7 @@ __global__ void __launch_bounds__(BX * BY) k_ff_unpack(Grid g, const float4* __r
 
 // out[rhs] = ||v|| of a float-float vector (one kernel, last-block finish).
 __global__ void __launch_bounds__(BX * BY) k_ff_norm(Grid g, const float4* __restrict__ v, double* __restrict__ out,
-                                                     double* partial, unsigned* tickets) {
+                                                     double* partial, unsigned* tickets, float* rscale) {
   __shared__ double sh[NVMAX * 32];
   FF_NODE
   double a[1] = {0.0};
@@ -181,8 +184,10 @@ __global__ void __launch_bounds__(BX * BY) k_ff_norm(Grid g, const float4* __res
   double s[1];
   if (reduce_last<1, double>(a, s, sh, partial, tickets, rhs, gridDim.x * gridDim.y,
                              blockIdx.y * gridDim.x + blockIdx.x) &&
-      threadIdx.x == 0 && threadIdx.y == 0)
+      threadIdx.x == 0 && threadIdx.y == 0) {
     out[rhs] = sqrt(s[0]);
+    rscale[2 * rhs] = rscale[2 * rhs + 1] = inv_pow2(out[rhs]);
+  }
 }
 
 // Per-node float-float diagonal w (4/h^2 - k^2) for variable k (dense).
@@ -220,8 +225,9 @@ void launch_ff_resid_cast_stop(const Grid& g, const FFConsts& K, const double* k
                                                                 (const float4*)b, r32, c, count);
 }
 
-void launch_ff_update(const Grid& g, void* x, const float2* e, int B, const int* active, cudaStream_t s) {
-  k_ff_update<<<ff_grid(g, B), dim3(BX, BY), 0, s>>>(g, (float4*)x, e, active);
+void launch_ff_update(const Grid& g, void* x, const float2* e, int B, const int* active, const float* rscale,
+                      cudaStream_t s) {
+  k_ff_update<<<ff_grid(g, B), dim3(BX, BY), 0, s>>>(g, (float4*)x, e, active, rscale);
 }
 
 void launch_ff_pack(const Grid& g, const double2* user, void* v, int B, int conj, cudaStream_t s) {
@@ -233,8 +239,8 @@ void launch_ff_unpack(const Grid& g, const void* v, double2* user, int B, int co
 }
 
 void launch_ff_norm(const Grid& g, const void* v, int B, double* out, double* partial, unsigned* tickets,
-                    cudaStream_t s) {
-  k_ff_norm<<<ff_grid(g, B), dim3(BX, BY), 0, s>>>(g, (const float4*)v, out, partial, tickets);
+                    float* rscale, cudaStream_t s) {
+  k_ff_norm<<<ff_grid(g, B), dim3(BX, BY), 0, s>>>(g, (const float4*)v, out, partial, tickets, rscale);
 }
 
 }  // namespace hmg

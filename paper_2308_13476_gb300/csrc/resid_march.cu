@@ -101,6 +101,7 @@ template <bool VK> struct RmMarch {
   float2* r;              // this lane's first node of row j
   int pitch, n1;
   bool ok0, ok1, out0, out1;
+  float gs;                   // factor of the stored residual (Ctl::rscale)
   double ih2, dc;
   double2 X[2][2], Q[2][2];   // rows in flight: x of rows j + 1, j + 2 and b of rows j, j + 1
   double D[2][2];             // VK: k of rows j, j + 1
@@ -139,9 +140,10 @@ template <bool VK> struct RmMarch {
     for (int n = 0; n < 2; ++n)
       f[n] = cast2(make_double2(fma(ih2, s[n].x, fma(-d[n], xc[n].x, q[n].x)),
                                 fma(ih2, s[n].y, fma(-d[n], xc[n].y, q[n].y))));
-    if (out0 && out1) *reinterpret_cast<float4*>(r) = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
-    else if (out0) r[0] = f[0];
-    else if (out1) r[1] = f[1];
+    const float2 o[2] = {mul2(bc2(gs), f[0]), mul2(bc2(gs), f[1])};
+    if (out0 && out1) *reinterpret_cast<float4*>(r) = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+    else if (out0) r[0] = o[0];
+    else if (out1) r[1] = o[1];
     r += pitch;
     const float t0 = fmaf(f[0].x, f[0].x, f[0].y * f[0].y), t1 = fmaf(f[1].x, f[1].x, f[1].y * f[1].y);
     sum.add((out0 ? t0 : 0.f) + (out1 ? t1 : 0.f));
@@ -162,6 +164,7 @@ template <bool A2, bool VK> __device__ __forceinline__ void rm_body(const RmA& a
   const double2* xs = a.x + off;
   const double2* bs = a.b + off;
   float2* rs = a.r32 + off;
+  const float gs = a.c.rscale[2 * rhs + 1];
   CSum sum;
   if (w < a.m.ns * a.m.nch) {
     const int strip = w % a.m.ns, i = strip * RMS + 2 * lane;
@@ -171,6 +174,7 @@ template <bool A2, bool VK> __device__ __forceinline__ void rm_body(const RmA& a
     p.ok1 = i + 1 <= g.nx;
     p.out0 = lane > 0 && i < g.nx;
     p.out1 = lane < 31 && i + 1 < g.nx;
+    p.gs = gs;
     p.pitch = g.pitch;
     p.n1 = g.nx + 1;
     p.ih2 = a.op.c.inv_h2;
@@ -224,7 +228,7 @@ template <bool A2, bool VK> __device__ __forceinline__ void rm_body(const RmA& a
       }
       const int at = g.at(i, j);
       const float2 f = cast2(sub<double>(bs[at], op.apply(xs, at, g.pitch, i, j)));
-      rs[at] = f;
+      rs[at] = mul2(bc2(gs), f);
       sum.add(fmaf(f.x, f.x, f.y * f.y));
     }
   }
@@ -232,7 +236,7 @@ template <bool A2, bool VK> __device__ __forceinline__ void rm_body(const RmA& a
   double v[1];
   __syncwarp();
   if (reduce_last<1, float>(a0, v, sh, a.c.partial, a.c.tickets, rhs, a.m.blocks(), blk) && threadIdx.x == 0)
-    stop_update(a.c, rhs, v[0], a.count);
+    stop_update(a.c, rhs, v[0], a.count, gs);
 }
 
 template <bool A2, bool VK>   // the k field's rows in flight take the registers of one block

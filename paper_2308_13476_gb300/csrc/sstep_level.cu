@@ -328,6 +328,7 @@ struct SuA {
   float iscale, sigma;
   const double* st;
   const int* active;
+  const float* rscale; // OUT: x' is divided by rscale[2 rhs]
 };
 
 // Z: x is zero (not read).  NR: the residual too.
@@ -343,6 +344,8 @@ __device__ __forceinline__ void sl_update_body(const SuA& a, uint3 blk, int rhs)
 #pragma unroll
   for (int k = 0; k < 3; ++k) y[k] = make_float2(S[2 * k], S[2 * k + 1]);
   if constexpr (NR) ss_residual_coef(y, a.iscale, a.sigma, c);
+  [[maybe_unused]] double ig = 1.0;
+  if constexpr (OUT) ig = f64_from_f32(rcp_pow2(a.rscale[2 * rhs]));
   for (int q = 0, j = blk.y * BY * g.ry + threadIdx.y; q < g.ry; ++q, j += BY) {
     if (j > g.ny) break;
     const long long p = off + g.at(i0, j);
@@ -369,8 +372,8 @@ __device__ __forceinline__ void sl_update_body(const SuA& a, uint3 blk, int rhs)
       for (int n = 0; n < 2; ++n)
         if (n < nv) {
           double2 o = a.outer[p + n];
-          o.x += f64_from_f32(x.v[n].x);
-          o.y += f64_from_f32(x.v[n].y);
+          o.x = fma(ig, f64_from_f32(x.v[n].x), o.x);
+          o.y = fma(ig, f64_from_f32(x.v[n].y), o.y);
           a.outer[p + n] = o;
         }
     } else {
@@ -417,7 +420,7 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
   float2* const u2 = (float2*)gb.u[2];
   float2* const w = (float2*)gb.w;
   SlA a{g, nullptr, b, nullptr, u1, nullptr, gb.scale, gb.sigma, gb.st, gb.partial, gb.tickets, active, B};
-  SuA u{g, x, nullptr, u1, u2, w, u0, gb.outer, 1.f / gb.scale, gb.sigma, gb.st, active};
+  SuA u{g, x, nullptr, u1, u2, w, u0, gb.outer, 1.f / gb.scale, gb.sigma, gb.st, active, gb.rscale};
   // apply(mode, v, out): one application of this level's kernels
   auto steps = [&](auto apply) {
     const float2* r = u0;
@@ -531,7 +534,7 @@ void gmres_smooth_ss_rag(const std::vector<RagLevel<float>>& v, int nu, bool wan
         rag_launch<SuA>(n, kern, dim3(BX, BY), 0, s, [&](int q, SuA& a, int& gx, int& gy) {
           const RagLevel<float>& L = v[q];
           a = SuA{L.g, L.x, (float2*)L.gb.u[0], (float2*)L.gb.u[1], (float2*)L.gb.u[2], (float2*)L.gb.w,
-                  (float2*)L.gb.u[0], nullptr, 1.f / L.gb.scale, L.gb.sigma, L.gb.st, L.active};
+                  (float2*)L.gb.u[0], nullptr, 1.f / L.gb.scale, L.gb.sigma, L.gb.st, L.active, nullptr};
           const dim3 d = pack_blocks(L.g, 1);
           gx = d.x;
           gy = d.y;

@@ -54,6 +54,7 @@ struct SmA {
   unsigned* tickets;
   const int* active;
   int nblk;            // blocks per right-hand side
+  const float* rscale; // update into outer: x' is divided by rscale[2 rhs]
 };
 
 // Warp modes: 0 interior strips (branch-free five-point stencil), 1 strips
@@ -257,6 +258,7 @@ template <int MODE, bool Z, bool VK, bool OUT> struct SUpd : SMarch<MODE, Z, VK>
   const double2* xs; // and of the row 4 steps ahead, staged with the input rows (fields NF, NF + 1 of the ring)
   int rs;            // that row, counted from j0
   int nv;            // nodes of this lane to write (0: none)
+  double ig;         // OUT: 1 / rscale
   float2 y[3];
   __device__ __forceinline__ void stage64(uint32_t slot) {
 #pragma unroll
@@ -295,7 +297,7 @@ template <int MODE, bool Z, bool VK, bool OUT> struct SUpd : SMarch<MODE, Z, VK>
           if (n < nv) {
             const double2 o = *reinterpret_cast<const double2*>(
                 __cvta_shared_to_generic(this->m.sh + this->m.half + (M::NF + n) * RING + S * 512));
-            x64[n] = make_double2(o.x + f64_from_f32(u[n].x), o.y + f64_from_f32(u[n].y));
+            x64[n] = make_double2(fma(ig, f64_from_f32(u[n].x), o.x), fma(ig, f64_from_f32(u[n].y), o.y));
           }
       } else {
         if (nv == 2) *reinterpret_cast<float4*>(xo) = make_float4(u[0].x, u[0].y, u[1].x, u[1].y);
@@ -378,6 +380,7 @@ __device__ __forceinline__ void upd_run(const SmA& a, int strip, int j0, int j1,
   p.xo = a.xo + at;
   p.x64 = a.outer + at;
   p.xs = p.x64;
+  if constexpr (OUT) p.ig = f64_from_f32(rcp_pow2(a.rscale[2 * rhs]));
   p.rs = -SHW - 2 - SMarch<MODE, Z, VK>::D;
   p.m.prime([&](uint32_t slot) {
     if constexpr (OUT) p.stage64(slot);
@@ -475,7 +478,7 @@ long long ss_march_blocks(const Grid& g, int B) { return cdiv(ss_geo(g, B).nrec(
 float2* gmres_smooth_ss_march(const Grid& g, const OpView<float>& opv, float2* x, float2* xt, const float2* b, int nu,
                               int B, const int* active, const GmresBufs& gb, cudaStream_t s) {
   SmA a{g, ss_geo(g, B), Op0<float>{opv.c0, opv.kf, g.nx, g.ny}, gb.scale, gb.sigma, x, b, xt, gb.outer,
-        gb.st, gb.partial, gb.tickets, active, 0};
+        gb.st, gb.partial, gb.tickets, active, 0, gb.rscale};
   a.nblk = cdiv(a.mg.nrec(), SWB);
   const dim3 grid(a.nblk, 1, B);
   auto steps = [&](auto vk, auto a2) {
@@ -509,7 +512,7 @@ void gmres_smooth_ss_march_rag(std::vector<RagLevel<float>>& v, int nu, cudaStre
   for (int q = 0; q < n; ++q) {
     RagLevel<float>& L = v[q];
     A[q] = SmA{L.g, ss_geo(L.g, 1), Op0<float>{L.op.c0, L.op.kf, L.g.nx, L.g.ny}, L.gb.scale, L.gb.sigma, L.x, L.b,
-               L.xt, nullptr, L.gb.st, L.gb.partial, L.gb.tickets, L.active, 0};
+               L.xt, nullptr, L.gb.st, L.gb.partial, L.gb.tickets, L.active, 0, nullptr};
     A[q].nblk = cdiv(A[q].mg.nrec(), SWB);
   }
   auto launch = [&](auto kern) {
