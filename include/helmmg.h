@@ -101,8 +101,10 @@ typedef struct {
                        kernels, which then also form the residual before the
                        restriction (needs fuse = 1): 1 = always, 0 = never (the
                        node-parallel kernels; same results to rounding),
-                       -1 = the Kronecker-form levels and the complex64 fine
-                       level; the complex128 fine level runs node-parallel
+                       -1 = the Kronecker-form levels (weighted Jacobi: those
+                       with enough nodes over all right-hand sides) and the
+                       complex64 fine level; the complex128 fine level runs
+                       node-parallel
                        (the FP64 pipe bounds it, and the marches' halos cost
                        more there than the passes that they save)            */
   int krylov;       /* 0 = the stand-alone cycle iteration (the paper's method);

@@ -281,6 +281,19 @@ static bool use_march(const mg_ctx* c, int l) {
   return c->opt.march == 1 || c->lev[l].kind >= 4;
 }
 
+// Whether a Kronecker-form level's weighted-Jacobi sweeps run as column marches:
+// from JK_MARCH nodes over all right-hand sides on.  A march's warp walks at
+// least eight rows and its halo one after the other, so a small level is quicker
+// node-parallel.  FP64 V(2,2), every level as grid-wide kernels, us per cycle,
+// marched everywhere / by this rule / never: 65^2 652 / 491 / 487, 8 x 257^2
+// 1240 / 1098 / 1191, 8 x 513^2 2257 / 2114 / 2621; complex64 8 x 257^2
+// 257 / 233 / 233, 8 x 1025^2 928 / 910 / 1044.
+constexpr long long JK_MARCH = 40000;
+static bool jacobi_march(const mg_ctx* c, int l) {
+  if (!use_march(c, l) || c->lev[l].kind < 4) return false;
+  return c->opt.march == 1 || c->lev[l].plane * c->B >= JK_MARCH;
+}
+
 // Whether level l's complex64 GMRES(3) steps run as the s-step row marches:
 // the fine level whenever marches are allowed.  They need no size threshold:
 // on one 1025^2 right-hand side a step takes 31 us against the node-parallel
@@ -352,10 +365,10 @@ template <class T> struct Emit {
         std::swap(cur[l], oth[l]);
       }
     } else if (c->opt.smoother == 0) {
-      // a zero iterate needs no application, and a Kronecker-form level takes
-      // its sweeps as column marches (a third of OpK::apply's arithmetic): 8 x
-      // 257^2, radius 2, 17.1 -> 4.6 and 9.8 us, 129^2, radius 3, 10.9 -> 3.6 and 10.3 us
-      const bool march = c->opt.fuse && op.kind >= 4 && use_march(c, l);
+      // a zero iterate needs no application, and a large enough Kronecker-form
+      // level takes its sweeps as column marches (a third of OpK::apply's
+      // arithmetic): 8 x 257^2, radius 2, 17.1 -> 4.6 and 9.8 us
+      const bool march = jacobi_march(c, l);
       for (int q = 0; q < nu; ++q) {
         if (z && q == 0) launch_jacobi<T>(g, op, nullptr, V.b, oth[l], c->B, c->active, s);
         else if (march) launch_kron_jacobi<T>(g, op, cur[l], V.b, oth[l], c->B, c->active, c->opt.kron_chunk, s);
