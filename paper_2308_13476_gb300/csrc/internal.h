@@ -291,8 +291,9 @@ struct ClStep {
 template <class T> struct ClLev {
   int nx, ny, n1, rp;         // intervals, nodes per row, rows per block
   int kind;                   // as OpView::kind
-  unsigned magic;             // q / n1 = umulhi(q, magic) for the slab's nodes
+  unsigned magic, mrp;        // q / n1 = umulhi(q, magic) for the slab's nodes, j / rp = umulhi(j, mrp) for the rows
   int ox, ob, od;             // shared memory (elements): iterate, right-hand side, inverse diagonal (-1: none)
+  int ost;                    // stored stencil of the slab, [(2R+1)^2][rp n1] (-1: read from L2)
   int ogx, owx, ohy, owy;     // Kronecker factors: x rows transposed to [2R+1][n1], the slab's y rows
   T scale, sigma;             // s-step basis (sstep.cuh)
   T w0, w1, w2;               // transfers between this level and the next (Xfer)
