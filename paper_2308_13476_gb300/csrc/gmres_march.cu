@@ -498,7 +498,7 @@ template <class T> MGeo march_geo(const Grid& g, int B) {
   MGeo m;
   m.fill(g.nx, g.ny, SW, 32 * NP, 2, 3);
   const int inner_rows = g.ny - 5;
-  const long long want = 152LL * 48;   // warps to fill the GPU a few times over
+  const long long want = (long long)device_sms() * 48;   // warps to fill the GPU a few times over
   int ch = 64;
   while (ch > 8 && (long long)m.nstrips * cdiv(inner_rows, ch) * B < want) ch /= 2;
   m.chunks(ch);

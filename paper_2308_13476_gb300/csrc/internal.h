@@ -72,6 +72,19 @@ template <class T> void launch_apply(const Grid& g, const OpView<T>& op, const c
 // x = null: x is zero (the sweep is xout = (omega diag A)^{-1} b).
 template <class T> void launch_jacobi(const Grid& g, const OpView<T>& op, const cx<T>* x, const cx<T>* b,
                                       cx<T>* xout, int B, const int* active, cudaStream_t s);
+// Streaming multiprocessors of the device, for the launches' geometry: asked for
+// once, so that a buffer sized by a geometry and the launches that fill it
+// always go by one number.
+inline int device_sms() {
+  static const int n = [] {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaGetLastError();
+    return sms > 0 ? sms : 1;
+  }();
+  return n;
+}
 // Per-solve control block of the stopping test (device arrays, one entry per
 // RHS unless noted).  tolp = {tol, divergence threshold}; partial/tickets are
 // the scratch of the fused reductions (reduce_last).

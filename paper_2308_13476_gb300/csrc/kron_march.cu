@@ -188,12 +188,10 @@ __global__ void __launch_bounds__(KW * 32) km_arn_a_rag(const __grid_constant__ 
 // its time (8 x 129^2, radius 3: 86 -> 56 us with one block of 9 rows per SM).
 template <class T, int R> long long kron_capacity() {
   static const long long cap = [] {
-    int dev = 0, sms = 1, per = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per = 1;
     if (sizeof(T) == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, km_arn_a<T, R, 2>, KW * 32, 0);
     cudaGetLastError();
-    return (long long)std::max(per, 1) * std::max(sms, 1);
+    return (long long)std::max(per, 1) * device_sms();
   }();
   return cap;
 }

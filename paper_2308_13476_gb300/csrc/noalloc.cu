@@ -31,7 +31,7 @@ namespace {
 constexpr int NA_TILE = 32;                           // grids are accepted by their count of 32 x 32 tiles
 constexpr int NA_MAX_BLOCKS = 16384;                  // -> at most 16.7 M nodes
 constexpr int NA_NT = 256;                            // threads per block
-constexpr int NA_RESIDENT = 152 * 6;                  // blocks of the one-node form that run at once
+constexpr int NA_RESIDENT = 6;                        // blocks of the one-node form that run at once on an SM
 constexpr int NA_MAX_DEVICES = 64;
 }  // namespace
 
@@ -176,7 +176,7 @@ extern "C" mg_status mg_residual_norm_static(int nx, int ny, double h, const dou
   const double dc = 4.0 * op.c.inv_h2 - op.c.k * op.c.k;
   const double2 *xv = (const double2*)x, *bv = (const double2*)b;
   auto launch = [&](auto kern, int ry) { kern<<<cdiv(nodes, NA_NT * ry), NA_NT, 0, s>>>(op, nodes, dc, xv, bv, scratch, out); };
-  if (cdiv(nodes, NA_NT) <= NA_RESIDENT) launch(k_field ? k_resnorm_dense<1, true> : k_resnorm_dense<1, false>, 1);
+  if (cdiv(nodes, NA_NT) <= NA_RESIDENT * device_sms()) launch(k_field ? k_resnorm_dense<1, true> : k_resnorm_dense<1, false>, 1);
   else launch(k_field ? k_resnorm_dense<4, true> : k_resnorm_dense<4, false>, 4);
   e = cudaGetLastError();
   if (e != cudaSuccess) {

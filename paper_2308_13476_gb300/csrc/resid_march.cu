@@ -54,7 +54,7 @@ RmGeo rm_geo(const Grid& g, int B) {
     t.ch = ch;
     t.nch = cdiv(g.ny - 1, ch);
     t.nw = t.ns * t.nch + cdiv(m.nring, 32 * RMN);
-    const long long cost = ((long long)t.blocks() * B + 151) / 152 * (2 * ch + 3) + (2 * ch + 3);
+    const long long cost = cdiv((long long)t.blocks() * B, (long long)device_sms()) * (2LL * ch + 3) + (2 * ch + 3);
     if (best < 0 || cost <= best) {
       best = cost;
       m = t;

@@ -304,12 +304,10 @@ __global__ void __launch_bounds__(KW * 32) kl_apply_rag(const __grid_constant__ 
 // chunk height, since the Gram march takes twice the registers of the others.
 template <int R, int MODE> long long kl_capacity() {
   static const long long cap = [] {
-    int dev = 0, sms = 1, per = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kl_apply<R, MODE>, KW * 32, 0);
     cudaGetLastError();
-    return (long long)std::max(per, 1) * std::max(sms, 1);
+    return (long long)std::max(per, 1) * device_sms();
   }();
   return cap;
 }
@@ -464,7 +462,7 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
   // in blocks of 512 threads once blocks of 256 would be more than two per SM
   // (half as many records for the last block to add).  The other operators
   // have nothing to share.
-  const long long nb = (long long)cdiv(g.nx + 1, BX * 2) * cdiv(g.ny + 1, BY);
+  const long long nb = (long long)cdiv(g.nx + 1, BX * 2) * cdiv(g.ny + 1, BY), fill = 2LL * device_sms();
   with_op<float>(opv, g.nx, g.ny, [&](auto op) {
     using Op = decltype(op);
     auto go = [&](auto rb) {
@@ -489,9 +487,9 @@ void gmres_smooth_ss(const Grid& g, const OpView<float>& opv, bool march, float2
           sl_one<R, MODE, NY><<<grd, blk, 0, s>>>(a, op);
         });
       };
-      if (B >= 4 && nb * cdiv(B, 4) >= 304) go(std::integral_constant<int, 4>{});
-      else if (B >= 2 && nb * cdiv(B, 2) >= 304) go(std::integral_constant<int, 2>{});
-      else if (sl_blocks(g) * B > 304) one(std::integral_constant<int, 16>{});
+      if (B >= 4 && nb * cdiv(B, 4) >= fill) go(std::integral_constant<int, 4>{});
+      else if (B >= 2 && nb * cdiv(B, 2) >= fill) go(std::integral_constant<int, 2>{});
+      else if (sl_blocks(g) * B > fill) one(std::integral_constant<int, 16>{});
       else one(std::integral_constant<int, 8>{});
     } else {
       go(std::integral_constant<int, 1>{});

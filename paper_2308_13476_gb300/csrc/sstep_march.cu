@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(SWB * 32, 4) ss_update_rag(const __grid_consta
 MGeo ss_geo(const Grid& g, int B) {
   MGeo m{};
   m.fill(g.nx, g.ny, SSW, 64, SHW, SBR);
-  const long long resident = 152LL * 4;
+  const long long resident = 4LL * device_sms();
   long long best = -1;
   int bch = 8;
   for (int ch = 4; ch <= 256; ch += 4) {

@@ -26,3 +26,12 @@ def test_warp_exchanges_name_their_lanes():
     gives those that happen to have converged, which the language leaves open
     after a divergent branch."""
     assert [f for f, s in _sources().items() if "__activemask" in s] == []
+
+
+def test_launch_geometry_asks_the_device_for_its_size():
+    """No choice of a launch's geometry rests on one chip's number of streaming
+    multiprocessors (152, or a small multiple of it) written into the code."""
+    sizes = {152 * m + d for m in (1, 2, 3, 4, 6, 8) for d in (-1, 0)}
+    found = {f: sorted({int(v) for v in re.findall(r"(?<![\w.])(\d+)(?:[uUlL]*)(?![\w.])", s)} & sizes)
+             for f, s in _sources().items()}
+    assert {f: v for f, v in found.items() if v} == {}
