@@ -182,15 +182,17 @@ __global__ void __launch_bounds__(KW * 32) km_arn_a_rag(const __grid_constant__ 
 }
 
 // Blocks that share the device's time in the choice of the chunk height
-// (kron_geo).  complex64: the blocks of the level's heaviest march (km_arn_a<T,
-// R, 2>) resident at once.  complex128: one per SM, because one warp per
-// scheduler already fills the FP64 pipe, so a second block on an SM doubles
-// its time (8 x 129^2, radius 3: 86 -> 56 us with one block of 9 rows per SM).
-template <class T, int R> long long kron_capacity() {
+// (kron_geo).  complex64: the blocks of the launched march (residual or Jacobi
+// sweep) resident at once.  complex128: one per SM, because one warp per
+// scheduler already fills the FP64 pipe, so a second block on an SM doubles its
+// time (8 x 129^2, radius 3: 86 -> 56 us with one block of 9 rows per SM).
+template <class T, int R, int OUT> long long kron_capacity() {
   static const long long cap = [] {
     int per = 1;
-    if (sizeof(T) == 4) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, km_arn_a<T, R, 2>, KW * 32, 0);
-    cudaGetLastError();
+    if constexpr (sizeof(T) == 4) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, km_init<T, R, OUT>, KW * 32, 0);
+      cudaGetLastError();
+    }
     return (long long)std::max(per, 1) * device_sms();
   }();
   return cap;
@@ -220,7 +222,7 @@ void gmres_smooth_kron(const Grid& g, const OpView<T>& opv, cx<T>* x, const cx<T
   double* st = gb.st;
   auto run = [&](auto op, auto rad) {
     constexpr int R = decltype(rad)::value;
-    const KGeo kg = kron_geo(g, B, R, kron_capacity<T, R>(), gb.kron_ch);
+    const KGeo kg = kron_geo(g, B, R, kron_capacity<T, R, KM_NORM>(), gb.kron_ch);
     const dim3 grd(cdiv((long long)kg.ncw * kg.nchunks, KW), 1, B);
     for (int step = 0; step < nu; ++step) {
       // a zero x: u0 = b itself (read-only in every later pass)
@@ -249,7 +251,7 @@ void kron_pass(const Grid& g, const OpView<T>& opv, const cx<T>* x, const cx<T>*
                int kron_ch, cudaStream_t s) {
   auto run = [&](auto op, auto rad) {
     constexpr int R = decltype(rad)::value;
-    const KGeo kg = kron_geo(g, B, R, kron_capacity<T, R>(), kron_ch);
+    const KGeo kg = kron_geo(g, B, R, kron_capacity<T, R, OUT>(), kron_ch);
     const dim3 grd(cdiv((long long)kg.ncw * kg.nchunks, KW), 1, B);
     km_init<T, R, OUT><<<grd, KW * 32, 0, s>>>(g, kg, op, x, b, r, nullptr, nullptr, nullptr, active);
   };
@@ -283,7 +285,7 @@ void gmres_smooth_kron_rag(const std::vector<RagLevel<T>>& v, int nu, cudaStream
       const RagLevel<T>& L = v[q];
       const OpView<T>& o = L.op;
       const OpK<T, R> op = kron_op<T, R>(o, L.g.nx, L.g.ny);
-      const KGeo kg = kron_geo(L.g, 1, R, kron_capacity<T, R>(), L.gb.kron_ch);
+      const KGeo kg = kron_geo(L.g, 1, R, kron_capacity<T, R, KM_NORM>(), L.gb.kron_ch);
       A[q] = KmA<T, R>{L.g, kg, op, L.x, L.b, (cx<T>*)L.gb.u[0], (cx<T>*)L.gb.u[1], (cx<T>*)L.gb.u[2],
                        (cx<T>*)L.gb.w, L.gb.st, L.gb.partial, L.gb.tickets, L.active};
     }
