@@ -489,21 +489,18 @@ def run_ours(a):
     # roofline of the dominant kernel, timed live with CUDA events on the library's stream
     what = 5 if a.krylov else (0 if a.smoother == "jacobi" else 4)
     kms, kbytes = s.profile(what, 0, reps=20)
-    if what == 4 and a.precision != "fp64":
-        # mg_profile counts the 13 vector passes of the Arnoldi form; the two
-        # s-step marches that run read x and b twice and write x once
-        kbytes *= 5.0 / 13.0
+    passes, form = gmres_step_form(a.precision, tuned["march"])
+    if what == 4:   # the passes that run (mg_profile counts the Arnoldi form's)
+        kbytes = passes * (16 if a.precision == "fp64" else 8) * float(N) * a.batch
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     peak = peaks.get("hbm_gbs", 6800.0)
     peak_src = "measured hbm_gbs" if "hbm_gbs" in peaks else "fallback 6800 GB/s (no measured peaks file)"
     achieved = kbytes / (kms * 1e-3) / 1e9
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": step_traffic(a, what),
+            "traffic": step_traffic(a, what) if what != 4 or passes == 5 else None,
             "kernel": ({0: "level-0 weighted-Jacobi sweep",
-                        4: ("level-0 GMRES(3) smoothing step: 4 row-march passes + update, 16 vector passes"
-                            if a.precision == "fp64" else
-                            "level-0 GMRES(3) smoothing step in s-step form: two row marches, 5 vector passes"),
+                        4: f"level-0 GMRES(3) smoothing step: {form}, {passes} vector passes",
                         5: f"last FGMRES({a.krylov}) Arnoldi step (MGS-coefficient pass + new-vector pass, "
                            f"{2 * a.krylov + 1} FP64 and 3 cycle-precision vector passes)"}[what]) +
                       f" ({'complex128' if a.precision == 'fp64' else 'complex64'}), "
@@ -595,6 +592,17 @@ def run_ours(a):
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
+
+
+def gmres_step_form(precision, march):
+    """Vector passes of one GMRES(3) step of the constant-k fine level from a
+    non-zero iterate, and the kernels that make them (the library's dispatch;
+    march: its option)."""
+    if precision == "fp64":   # Arnoldi form
+        return (16, "4 row-march passes + update") if march == 1 else (28, "8 node-parallel passes")
+    if march == 0:            # s-step form: residual 3, v_1 2, v_2 2, Gram sums 3, update 5
+        return 15, "s-step form, 5 node-parallel passes"
+    return 5, "s-step form, two row marches"   # x, b; x, b -> x'
 
 
 def step_traffic(a, what):
