@@ -451,7 +451,7 @@ static Ctl ctl(const mg_ctx* c) {
 }
 
 // Records the steps of one visit of level lc (the same recursion as
-// Emit::cycle) for the coarse-cycle interpreter.
+// Emit::cycle) for the cooperative interpreter.
 template <class T> struct Plan {
   mg_ctx* c;
   std::vector<cx<T>*> cur, oth;
@@ -797,8 +797,8 @@ template <class T> static mg_status profile_t(mg_ctx* h, int what, int level, in
 // The cycle of every problem of a ragged batch as one graph whose kernels are
 // single launches over all problems (ragged.cuh).  The recursion is the one
 // of Emit::cycle, run on the set of problems that visit a level: problems
-// whose coarse-cycle launch starts at this level take it here (one CTA per
-// problem), the others smooth, restrict, recurse gamma times, prolong and
+// whose coarse-cycle launch starts at this level take it here (one cluster
+// per problem), the others smooth, restrict, recurse gamma times, prolong and
 // smooth.  Every problem sees its own kernels in the order Emit gives them.
 template <class T> struct EmitR {
   mg_ctx* c;

@@ -77,27 +77,13 @@ template <class T> __device__ __forceinline__ cx<T> psub(cx<T> a, cx<T> b) {
   else return sub<T>(a, b);
 }
 
-// s a - sum_l c_l v_l (the Arnoldi vector of a pass).  complex64: the real
-// parts of the coefficients scale v_l in one packed accumulator and the
-// imaginary parts in another, which are joined once (packed instructions
-// need no component swap that way); complex128 in the scalar order.
+// s a - sum_l c_l v_l (the Arnoldi vector of a pass)
 template <class T, int L>
 __device__ __forceinline__ cx<T> scl_minus(T s, cx<T> a, const cx<T> (&c)[L], const cx<T> (&v)[L]) {
-  if constexpr (sizeof(T) == 4) {
-    float2 p = mul2(bc2(s), a), q = mul2(bc2(c[0].y), v[0]);
-    p = fma2(bc2(-c[0].x), v[0], p);
+  cx<T> u = scl<T>(s, a);
 #pragma unroll
-    for (int l = 1; l < L; ++l) {
-      p = fma2(bc2(-c[l].x), v[l], p);
-      q = fma2(bc2(c[l].y), v[l], q);
-    }
-    return make_float2(p.x + q.y, p.y - q.x);
-  } else {
-    cx<T> u = scl<T>(s, a);
-#pragma unroll
-    for (int l = 0; l < L; ++l) u = sub_mul<T>(u, c[l], v[l]);
-    return u;
-  }
+  for (int l = 0; l < L; ++l) u = sub_mul<T>(u, c[l], v[l]);
+  return u;
 }
 
 // IEEE 754 conversions between binary64 and binary32 in integer arithmetic.

@@ -2,7 +2,7 @@
 //
 // One persistent cooperative launch walks the host-recorded V/W schedule of
 // the levels lc..L-1 (the same steps as the cluster launch of
-// cluster.cu, the same recursion as the grid-wide driver, Sec. 3 of the
+// cluster.cuh, the same recursion as the grid-wide driver, Sec. 3 of the
 // paper), with every block of the GPU working on every step: the blocks are
 // split evenly over the right-hand sides (bpr blocks per RHS) and phases are
 // separated by a grid-wide barrier instead of kernel boundaries.  A norm or

@@ -25,7 +25,7 @@ constexpr int G_BRK = 71;   // 1 = stop (breakdown or beta == 0)
 // global memory, or Ts where one thread block owns the state (every stored
 // value is a Ts value, so both storages give the same results).  The summed
 // inputs v of the fin_* steps come in V: FP64 from the grid-wide sums, Ts
-// from the block sums of the coarse-cycle interpreter.
+// from the block sums of the coarse-cycle launches.
 //
 // The scalars sit on the serial path of every smoothing step (one thread,
 // every launch of the Arnoldi process waits for them), so their cost is the

@@ -290,7 +290,7 @@ struct CStep {
   void* p1;                 // destination (Jacobi, copy) or coarse correction (prolong)
 };
 
-// Coarse-cycle launch (cluster.cu): the levels lc..L-1 of one right-hand side
+// Coarse-cycle launch (cluster.cuh): the levels lc..L-1 of one right-hand side
 // in the shared memory of a cluster of C blocks, which walks a host-recorded
 // list of steps.
 constexpr int CL_MAXC = 16;      // blocks per cluster
@@ -334,7 +334,9 @@ template <class T> struct ClArgs {
   int ou, nu, oX, nX, ored, olev, smem;   // shared memory layout (elements; smem in bytes)
 };
 // Largest cluster (a power of two, at most CL_MAXC) of which B run at once, so
-// that no right-hand side waits for another's visit to end; 0: none.
+// that no right-hand side of the handle waits for another's visit to end; 0: none.
+// The handles of a ragged batch ask for their own B only: their clusters together
+// can be more than the device holds, and then take turns.
 template <class T> int cluster_size(int B);
 // Fills the layout of levels (nx, ny, kind set) into lv and a; false if a
 // slab does not fit in a block's shared memory.

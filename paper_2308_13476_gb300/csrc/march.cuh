@@ -1,5 +1,5 @@
-// Building blocks of the fine level's row marches (gmres_march.cu,
-// sstep_march.cu): a warp walks a strip of columns down a chunk of rows, with
+// Building blocks of the fine level's row marches (gmres_march.cu, complex128;
+// sstep_march.cu, complex64, which has its own stencil and staging): a warp walks a strip of columns down a chunk of rows, with
 // the rows it needs in registers, horizontal neighbours by shuffles and input
 // rows staged ahead through a per-lane cp.async ring.
 #pragma once
@@ -59,12 +59,6 @@ __device__ __forceinline__ Row<double> stage_read(const double2* p) {
 template <class T> struct SlotT { using type = double2; };
 template <> struct SlotT<float> { using type = float4; };
 
-__device__ __forceinline__ void mstore(float2* __restrict__ d, const Grid& g, int i, int j, const Row<float>& r) {
-  if (i + 1 <= g.nx)
-    *reinterpret_cast<float4*>(d + g.at(i, j)) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
-  else if (i <= g.nx)
-    d[g.at(i, j)] = r.v[0];
-}
 __device__ __forceinline__ void mstore(double2* __restrict__ d, const Grid& g, int i, int j, const Row<double>& r) {
   if (i <= g.nx) d[g.at(i, j)] = r.v[0];
 }
@@ -109,13 +103,8 @@ template <class T, int MD> struct MCtx {
         const int ik = MM<MD> == 2 ? min(max(in, 0), op.nx) : in;   // edge strips: k of an in-grid node
         const T k = op.kf ? op.kf[m * (op.nx + 1) + ik] : op.c.k;
         const T d = fma(-k, k, T(4) * op.c.inv_h2);
-        if constexpr (sizeof(T) == 4) {   // the same operations, both components per instruction
-          const float2 sn = add2(add2(xe, xw), add2(xn, xs));
-          r.v[n] = fma2(bc2(d), xp, mul2(bc2(-op.c.inv_h2), sn));
-        } else {
-          const T sr = (xe.x + xw.x) + (xn.x + xs.x), si = (xe.y + xw.y) + (xn.y + xs.y);
-          r.v[n] = mk<T>(fma(d, xp.x, -op.c.inv_h2 * sr), fma(d, xp.y, -op.c.inv_h2 * si));
-        }
+        const T sr = (xe.x + xw.x) + (xn.x + xs.x), si = (xe.y + xw.y) + (xn.y + xs.y);
+        r.v[n] = mk<T>(fma(d, xp.x, -op.c.inv_h2 * sr), fma(d, xp.y, -op.c.inv_h2 * si));
         if (MM<MD> == 2) {   // rows are interior here; columns 0 and nx take the
                          // boundary row of Op0::apply5, columns off the grid zero
           const bool bcol = in == 0 || in == op.nx, inside = in >= 0 && in <= op.nx;

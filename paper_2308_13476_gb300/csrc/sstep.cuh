@@ -11,13 +11,15 @@
 // scale (about the inverse of the level's diagonal) keeps the powers in
 // range; sigma = 1 on the fine level, where scale A has its spectrum around
 // 1, keeps the basis well conditioned (median condition of the scaled normal
-// matrix 15 to 60 over a solve, against 2e3 to 1e4 with sigma = 0), and
-// sigma = 0 on the coarse levels (30 to 1e4 there either way).  The
-// least-squares minimum is flat, so an error e in z raises the residual only
-// by e^2: with FP32 scalars the cycle counts of constant-k, variable-k,
-// W-cycle and linear-transfer solves to 1e-6 and to 1e-11 are those of the
-// Arnoldi form.  complex128 cycles keep the Arnoldi form, whose iterates
-// follow modified Gram-Schmidt to rounding.
+// matrix over a solve 9 to 24, against 600 to 1100 with sigma = 0), and sigma = 0
+// the coarse levels' (17 to 45 on the first of them, against 2e4 to 7e4 with
+// sigma = 1; 30 to 2400 below).  The least-squares minimum is flat, so an error e
+// in z raises the residual only by e^2: with FP32 scalars the cycle counts of
+// constant-k, variable-k, W-cycle and linear-transfer solves to 1e-6 and to 1e-11
+// stay within 10 % (at least two) of the complex128 path's, which keeps the
+// Arnoldi form, whose iterates follow modified Gram-Schmidt to rounding.  The
+// cycle runs on its residual times a power of two near the inverse of its norm
+// (Ctl::rscale), so that the squares summed here stay in the float range.
 #pragma once
 #include "common.cuh"
 #include "gmres.cuh"

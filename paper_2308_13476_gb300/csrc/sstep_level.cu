@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(BX * BY) sl_apply(const __grid_constant__ SlA 
 // time), coefficients and v together, before the first multiply-add, and a
 // thread has half the loads and the launch twice the threads of the pair form.
 // Layered model 1281 x 449, one right-hand side, with the grouped loads of the
-// cluster launch (cluster.cu): 237 -> 162 ms.
+// cluster launch (cluster.cuh): 237 -> 162 ms.
 template <int R>
 __device__ __forceinline__ float2 stencil_node(const float2* st, long long plane, const float2* v, int pitch) {
   constexpr int K = 2 * R + 1, G = R == 2 ? 5 : 3;
